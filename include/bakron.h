@@ -222,8 +222,8 @@ int bakron_solve_with_grid(const void* W, int wdtype, int m, int n, int64_t ldw,
  * 256 samples accumulated afresh in the tensor core and added in fp32.
  * Otherwise kind::tf32 with operands split x = hi + lo and A B^T ~ hi hi^T +
  * hi lo^T + lo hi^T (bf16 rows are exact in tf32, so their lo MMAs are
- * skipped), each 32 samples accumulated afresh.  Only the lower-triangle
- * 128 x 128 blocks are computed.  Returns BAKRON_ERR_INVALID_ARG (bad
+ * skipped), each 32 samples accumulated afresh.  Only the blocks of the lower
+ * triangle are computed.  Returns BAKRON_ERR_INVALID_ARG (bad
  * pointer, k < 1, d outside 1..65536, strides), BAKRON_ERR_WORKSPACE, or the
  * device status (BAKRON_ERR_TIMEOUT if a bounded wait ran out).
  */

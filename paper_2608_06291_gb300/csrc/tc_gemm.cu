@@ -36,7 +36,6 @@
 // CTA winds down, draining its own TMA copies and MMAs (with a separate,
 // generous limit) before it frees TMEM.
 #include <cuda.h>
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 #include <stdint.h>
@@ -48,6 +47,7 @@
 #include "common.cuh"
 #include "profile.cuh"
 #include "tc_gemm.cuh"
+#include "tcgen05.cuh"
 
 namespace bakron {
 
@@ -86,7 +86,7 @@ static_assert(PAIR_STAGES * PAIR_STAGE_BYTES >= 8 * TILE_BYTES, "the epilogue st
 // X[:, S2] += E[:, S1] L^A[S2, S1]^T with S1 = tile columns [k, h) and S2 =
 // [h, l); it reads and writes like stage 2 (A = E in the M planes, B = L^A,
 // TMA reduce-add into X).
-enum Mode { MODE_DENSE = 0, MODE_STAGE1 = 1, MODE_STAGE2 = 2, MODE_GRAM = 3, MODE_COLS = 4 };
+enum Mode { MODE_DENSE = 0, MODE_STAGE1 = 1, MODE_STAGE2 = 2, MODE_COLS = 3 };
 
 struct TcParams {
   int mode;
@@ -100,29 +100,15 @@ struct TcParams {
   int64_t ldo;          // leading dimension of out_hi/out_lo/X (elements)
   int* status;
   long long spin_cycles;  // bound of the working waits (clock64 cycles)
-  // Gram mode: G <- beta G + alpha A B^T on the lower-triangle blocks, each
-  // entry (i, j <= i) < dreal written and mirrored to (j, i); a_exact /
-  // b_exact: that operand's lo plane is zero (skip its correction MMA)
-  float alpha, beta;
-  int dreal;
-  int a_exact, b_exact;
   unsigned long long* stamp;   // timeline stamp slot of the launch (null: none)
   int raster;                  // band stages: row blocks per launch-order group (>= 1)
 };
 
-// Kernel variants (compile time, so that the band products' issue loop
-// carries no Gram logic):
-//   V_BAND      band products and the dense diagnostic: 3xTF32, one K stage
-//               per TMEM accumulator, a slot freed by its accumulator's commit
-//   V_GRAM_TF32 Gram on tf32 hi/lo planes; a_exact / b_exact skip the MMAs
-//               of an operand whose lo plane is zero
-//   V_GRAM_BF16 Gram on bf16 planes: mapA2 / mapB2 are plain bf16 maps (64 x
-//               128 boxes), a ring slot holds one box of each (K = 64), the
-//               MMAs are kind::f16 (bf16 x bf16 products exact in fp32), and
-//               GRAM_KGROUP slots are summed in place per accumulator, each
-//               slot freed by its own commit to `empty`
-//   V_PAIR      band products and the dense diagnostic on CTA pairs (above)
-enum Variant { V_BAND = 0, V_GRAM_TF32 = 1, V_GRAM_BF16 = 2, V_PAIR = 3 };
+// Kernel variants (compile time):
+//   V_BAND  band products and the dense diagnostic: 3xTF32, one K stage per TMEM
+//           accumulator, a slot freed by its accumulator's commit
+//   V_PAIR  the same on CTA pairs (above)
+enum Variant { V_BAND = 0, V_PAIR = 1 };
 
 template <int V>
 struct Ring {
@@ -131,159 +117,10 @@ struct Ring {
   static constexpr uint32_t b_plane = pair ? TILE_BYTES / 2 : TILE_BYTES;   // one B plane
   static constexpr uint32_t stage_bytes = 2 * TILE_BYTES + 2 * b_plane;
 };
-constexpr int GRAM_KGROUP = 4;
-// Band products: K stages summed in place per TMEM accumulator (each group
-// restarts its accumulator; the epilogue adds the groups in fp32).  Two
-// stages per accumulator measured 1% faster per solve on GB300 but moved the
-// 4096^2 free-running objective from 8e-5 to 3e-4 of the fp64 solve's (an
-// earlier tie, then its cascade): one stage it is.
-constexpr int BAND_KGROUP = 1;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
-// Adds to the bytes the current phase waits for, without arriving.
-__device__ __forceinline__ void mbar_expect_tx_only(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Wait for the phase of `bar` with the given parity to complete, for at most
-// `limit` cycles.  Returns false on time-out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit) {
-  if (mbar_test(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (true) {
-    if (mbar_test(bar, parity)) return true;
-    if (clock64() - t0 > limit) return false;
-  }
-}
-
-// A hi/lo plane pair in one copy: a rank-3 box (32 columns, rows, 2 planes)
-// lands as the two planes one after the other (16 KiB each for 128 rows),
-// each in the 128-byte swizzled layout; one box instead of two halves the
-// TMA unit's per-box cost, which bounds the ring (measured on GB300: a 64 KiB
-// slot of four 16 KiB boxes takes 0.62 us, of two 32 KiB boxes 0.45 us).
-__device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* map, uint64_t* bar,
-                                              int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(0)
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
-                                            int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
-// 128 bytes, 8-row core groups 1024 bytes apart (SBO), version 1.
-// TMA store of a box from shared memory, and TMA reduce-add of a box into
-// global memory (fp32 add at L2), both tracked as a bulk group of the thread.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(y), "r"(smem_u32(src))
-               : "memory");
-}
-__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, const void* src, int x, int y) {
-  asm volatile(
-      "cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-          reinterpret_cast<uint64_t>(map)),
-      "r"(x), "r"(y), "r"(smem_u32(src))
-      : "memory");
-}
-__device__ __forceinline__ void bulk_commit_and_wait() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);            // start address
-  d |= (uint64_t)1 << 16;                             // leading byte offset (unused, 1)
-  d |= (uint64_t)(1024 >> 4) << 32;                   // stride byte offset
-  d |= (uint64_t)1 << 46;                             // descriptor version
-  d |= (uint64_t)2 << 61;                             // swizzle: 128 B
-  return d;
-}
-
-// Instruction descriptor: kind::tf32, D fp32, A and B tf32 K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
-  return (1u << 4)            // D format fp32
-         | (2u << 7)          // A format tf32
-         | (2u << 10)         // B format tf32
-         | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Instruction descriptor: kind::f16 with bf16 A and B (K-major), D fp32, M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4)            // D format fp32
-         | (1u << 7)          // A format bf16
-         | (1u << 10)         // B format bf16
-         | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
+// Each K stage restarts its TMEM accumulator and the epilogue adds the stages in
+// fp32: two stages summed in place measured 1% faster per solve on GB300 but moved
+// the 4096^2 free-running objective from 8e-5 to 3e-4 of the fp64 solve's (an
+// earlier tie, then its cascade).
 
 // ---- CTA-pair forms (cluster of two along y; rank 0 issues the MMAs)
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -382,25 +219,6 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// 32 lanes x 32 consecutive fp32 columns of TMEM into v (one per column) of
-// each thread; the values are valid only after tmem_wait_ld().
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // Output block and K range of this CTA.
 struct Block {
   int rb, cb;         // output block (128-row block, 128-col block)
@@ -477,7 +295,7 @@ __device__ __forceinline__ bool block_of(const TcParams& P, Block& b) {
   // the blocks with the longest K ranges first (they sit at high rows, and
   // in stage 2 at high columns): less of a tail when the grid runs in waves
   int bx = (int)blockIdx.x, by = (int)blockIdx.y;
-  if (P.mode != MODE_DENSE && P.mode != MODE_GRAM) {
+  if (P.mode != MODE_DENSE) {
     const int W = (int)gridDim.x, H = (int)gridDim.y;
     const int R = P.raster > 0 ? P.raster : RASTER_ROWS;
     const int L = by * W + bx, grp = L / (R * W), in = L - grp * R * W;
@@ -491,18 +309,6 @@ __device__ __forceinline__ bool block_of(const TcParams& P, Block& b) {
     b.cb = blockIdx.x;
     b.k0 = b.ok0 = 0;
     b.nk = b.onk = P.K / BK;
-    return true;
-  }
-  if (P.mode == MODE_GRAM) {
-    // block t of the lower triangle, row by row: t = rb (rb + 1) / 2 + cb, cb <= rb
-    const int t = blockIdx.x;
-    int rb = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-    while ((rb + 1) * (rb + 2) / 2 <= t) ++rb;
-    while (rb * (rb + 1) / 2 > t) --rb;
-    b.rb = rb;
-    b.cb = t - rb * (rb + 1) / 2;
-    b.k0 = b.ok0 = 0;
-    b.nk = b.onk = P.K / BK;   // K stages; the bf16 variant's K counts 128-byte rows of 64
     return true;
   }
   int cb_lo, cb_hi;
@@ -580,10 +386,9 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = (uint64_t*)(smem + NST * SB);
   uint64_t* full = bars;                 // [NST] smem stage loaded
-  uint64_t* empty = bars + NST;          // [NST] slot read by its MMAs (kgroup > 1 only;
-                                         // otherwise the slot's accF commit frees it)
-  uint64_t* accum = bars + 2 * NST;      // [1] every MMA of the CTA complete
-  uint64_t* accF = accum + 1;            // [NACC] accumulator holds a finished K stage
+  uint64_t* accum = bars + NST;          // [1] every MMA of the CTA complete
+  uint64_t* accF = accum + 1;            // [NACC] accumulator holds a finished K stage (and the
+                                         // stage's slot is free)
   uint64_t* accE = accum + 1 + NACC;     // [NACC] accumulator read out by the epilogue
   uint32_t* tmem_slot = (uint32_t*)(accum + 1 + 2 * NACC);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
@@ -611,10 +416,8 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapOl)) : "memory");
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) {
+    for (int s = 0; s < NST; ++s)
       mbar_init(&full[s], pair && rank == 0 ? 2 : 1);   // leader: its producer and the peer's
-      mbar_init(&empty[s], 1);
-    }
     mbar_init(accum, 1);
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&accF[a], 1);
@@ -660,7 +463,6 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
   };
   const int npre = blk.nk < NST ? blk.nk : NST;
   const bool a_static = P.mode != MODE_STAGE2 && P.mode != MODE_COLS;
-  constexpr bool bf16_ops = V == V_GRAM_BF16;
   // pairs: this CTA's A is zero (a fully out-of-range box) outside its own K
   // range; its half of B is rows 64 * rank .. of the column block
   auto a_row = [&](int kt) -> int {
@@ -672,11 +474,6 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
     for (int i = 0; i < npre; ++i) {
       unsigned char* st = smem + i * SB;
       const int kt = blk.k0 + i;
-      if constexpr (bf16_ops) {
-        mbar_expect_tx_only(&full[i], TILE_BYTES);
-        tma_load_2d(st, &mapA2, &full[i], kt * 2 * BK, blk.rb * BM);
-        continue;
-      }
       if constexpr (pair) {
         const uint32_t cb = cfull0 + (uint32_t)(i * 8);
         cmbar_expect_tx_only(cb, a_static ? 2 * TILE_BYTES : 2 * RG::b_plane);
@@ -699,8 +496,6 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
   stamp_begin(P.stamp);
   const long long drain = 4000000000LL;   // ~2 s at 2 GHz: wind-down bound
   const int nk = blk.nk;
-  constexpr int kgroup = V == V_GRAM_BF16 ? GRAM_KGROUP : (V == V_BAND ? BAND_KGROUP : 1);
-  const int ngroups = (nk + kgroup - 1) / kgroup;   // accumulator hand-overs
 
   if (warp == 0) {
     // ---------------------------------------------------------- producer
@@ -714,10 +509,7 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
       // cannot have moved on to stage j + NACC yet, which needs this load
       if (lane == 0 && i >= NST) {
         const int j = i - NST;
-        if constexpr (kgroup > 1)
-          ok = mbar_wait(&empty[s], (uint32_t)(j / NST) & 1u, P.spin_cycles);
-        else
-          ok = mbar_wait(&accF[j % NACC], (uint32_t)(j / NACC) & 1u, P.spin_cycles);
+        ok = mbar_wait(&accF[j % NACC], (uint32_t)(j / NACC) & 1u, P.spin_cycles);
       }
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok || *abort_flag) {
@@ -738,16 +530,6 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
       unsigned char *a_hi = st, *b_hi = st + 2 * TILE_BYTES, *b_lo = b_hi + RG::b_plane;
       const int kt = blk.k0 + i;            // K tile index (32 wide)
       const bool pre = i < npre;            // the factor operand is already on its way
-      if constexpr (bf16_ops) {             // one bf16 box per operand, 64 of K
-        if (lane == 0) {
-          mbar_expect_tx(&full[s], pre ? TILE_BYTES : 2 * TILE_BYTES);
-          if (!pre) tma_load_2d(a_hi, &mapA2, &full[s], kt * 2 * BK, blk.rb * BM);
-          tma_load_2d(b_hi, &mapB2, &full[s], kt * 2 * BK, blk.cb * BN);
-        }
-        __syncwarp();
-        issued = i + 1;
-        continue;
-      }
       const bool load_a = !(pre && a_static), load_b = !(pre && !a_static);
       if constexpr (pair) {
         // every box lands in full (an out-of-range one as zeros), so the
@@ -848,36 +630,33 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
     }
   } else if (warp == 1) {
     // --------------------------------------------------------- MMA issuer
-    // Each group of kgroup K stages (one stage in the band products, four of
-    // exact bf16 products in the Gram) accumulates afresh into accumulator
-    // (group mod NACC); the epilogue adds the groups in fp32 registers.  The
-    // tensor core's accumulation is not round-to-nearest, and its error grows
-    // with the number of MMAs summed in place; restarting every group bounds it.
+    // Each K stage accumulates afresh into accumulator (stage mod NACC); the
+    // epilogue adds the stages in fp32 registers.  The tensor core's accumulation
+    // is not round-to-nearest, and its error grows with the number of MMAs summed
+    // in place; restarting every stage bounds it.
     if (lane == 0 && pair && rank != 0) {
       // the peer: the leader's MMAs write this CTA's TMEM and read its shared
       // memory; its last commit arrives here too once they have completed
       if (nk == 0) mbar_arrive(accum);
       if (!mbar_wait(accum, 0, drain)) raise_status(status, BAKRON_ERR_TIMEOUT);
     } else if (lane == 0) {
-      const uint32_t idesc = idesc_tf32(pair ? 2 * BM : BM, BN), idesc_b = idesc_bf16(BM, BN);
+      const uint32_t idesc = idesc_tf32(pair ? 2 * BM : BM, BN);
       const uint64_t desc0 = smem_desc(smem_u32(smem));   // stage 0, A hi, K step 0
       for (int i = 0; i < nk; ++i) {
         const int s = i % NST;
         const uint32_t ph = (uint32_t)(i / NST) & 1u;
-        const int g = i / kgroup, a = g % NACC;     // accumulator group of this slot
-        const bool first = i % kgroup == 0;
-        const bool last = i % kgroup == kgroup - 1 || i == nk - 1;
-        // accumulator a was last used by group g - NACC: wait until it was read
+        const int a = i % NACC;     // accumulator of this stage
+        // accumulator a was last used by stage i - NACC: wait until it was read
         // out (the producer's and the epilogue's aborts surface here as time-outs)
         bool ok;
         if constexpr (pair)
           ok = mbar_wait_cluster(&full[s], ph, P.spin_cycles) &&
-               (!first || g < NACC ||
-                mbar_wait_cluster(&accE[a], (uint32_t)(g / NACC - 1) & 1u, P.spin_cycles));
+               (i < NACC ||
+                mbar_wait_cluster(&accE[a], (uint32_t)(i / NACC - 1) & 1u, P.spin_cycles));
         else
           ok = mbar_wait(&full[s], ph, P.spin_cycles) &&
-               (!first || g < NACC ||
-                mbar_wait(&accE[a], (uint32_t)(g / NACC - 1) & 1u, P.spin_cycles));
+               (i < NACC ||
+                mbar_wait(&accE[a], (uint32_t)(i / NACC - 1) & 1u, P.spin_cycles));
         if (!ok) {
           raise_status(status, BAKRON_ERR_TIMEOUT);
           abort_all();
@@ -890,32 +669,23 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
         const uint64_t dal = dah + (TILE_BYTES >> 4), dbh = dah + (2 * TILE_BYTES >> 4),
                        dbl = dbh + (RG::b_plane >> 4);
         const uint32_t d = tmem + (uint32_t)(a * BN);
-        if constexpr (bf16_ops) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)            // 16 bf16 = 32 bytes along K per MMA
-            mma_bf16(d, dah + 2 * kk, dbh + 2 * kk, idesc_b, (kk > 0 || !first) ? 1u : 0u);
-        } else if constexpr (pair) {
-#pragma unroll
-          for (int kk = 0; kk < BK / 8; ++kk) {
-            const uint64_t o = (uint64_t)(2 * kk);
-            mma_tf32_pair(d, dah + o, dbh + o, idesc, (kk > 0 || !first) ? 1u : 0u);
+        for (int kk = 0; kk < BK / 8; ++kk) {
+          const uint64_t o = (uint64_t)(2 * kk);   // 8 tf32 = 32 bytes along K inside the swizzle row
+          if constexpr (pair) {
+            mma_tf32_pair(d, dah + o, dbh + o, idesc, kk > 0 ? 1u : 0u);
             mma_tf32_pair(d, dah + o, dbl + o, idesc, 1u);
             mma_tf32_pair(d, dal + o, dbh + o, idesc, 1u);
-          }
-        } else {
-#pragma unroll
-          for (int kk = 0; kk < BK / 8; ++kk) {
-            const uint64_t o = (uint64_t)(2 * kk);   // 8 tf32 = 32 bytes along K inside the swizzle row
-            mma_tf32(d, dah + o, dbh + o, idesc, (kk > 0 || !first) ? 1u : 0u);
-            if (V == V_BAND || !P.b_exact) mma_tf32(d, dah + o, dbl + o, idesc, 1u);
-            if (V == V_BAND || !P.a_exact) mma_tf32(d, dal + o, dbh + o, idesc, 1u);
+          } else {
+            mma_tf32(d, dah + o, dbh + o, idesc, kk > 0 ? 1u : 0u);
+            mma_tf32(d, dah + o, dbl + o, idesc, 1u);
+            mma_tf32(d, dal + o, dbh + o, idesc, 1u);
           }
         }
         if constexpr (pair) {
-          if (last) mma_commit_pair(&accF[a]);   // both CTAs: the sum, and the slot
+          mma_commit_pair(&accF[a]);   // both CTAs: the sum, and the slot
         } else {
-          if constexpr (kgroup > 1) mma_commit(&empty[s]);   // the slot back to the producer
-          if (last) mma_commit(&accF[a]);  // the group's sum to the epilogue (kgroup 1: and the slot)
+          mma_commit(&accF[a]);        // the stage's sum to the epilogue, and the slot
         }
       }
       if (nk > 0) {  // tracks every MMA issued above
@@ -937,7 +707,7 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
 #pragma unroll
     for (int u = 0; u < EPI_COLS; ++u) acc[u] = 0.f;
     bool write = blk.own;
-    for (int i = 0; i < ngroups; ++i) {
+    for (int i = 0; i < nk; ++i) {
       const int a = i % NACC;
       // one lane waits; the decision is warp-uniform (tcgen05.ld is warp-collective)
       int ok = 1;
@@ -966,26 +736,7 @@ __device__ __forceinline__ void tc_body(const CUtensorMap& mapA2, const CUtensor
         else mbar_arrive(&accE[a]);
       }
     }
-    if (P.mode == MODE_GRAM) {
-      // entry (gi, gj <= gi) and its mirror (gj, gi); for a fixed u the warp's
-      // 32 lanes hold 32 consecutive gi, so the mirror stores are coalesced
-      const int64_t gi = (int64_t)blk.rb * BM + row;
-      const int64_t gj0 = (int64_t)blk.cb * BN + c0;
-      if (write && gi < P.dreal) {
-#pragma unroll
-        for (int u = 0; u < EPI_COLS; ++u) {
-          const int64_t gj = gj0 + u;
-          if (gj > gi) continue;          // also keeps gj < dreal
-          const float v = P.alpha * acc[u];
-          float* p = P.out_hi + gi * P.ldo + gj;
-          *p = P.beta == 0.f ? v : fmaf(P.beta, *p, v);
-          if (gj < gi) {
-            float* q2 = P.out_hi + gj * P.ldo + gi;
-            *q2 = P.beta == 0.f ? v : fmaf(P.beta, *q2, v);
-          }
-        }
-      }
-    } else if (P.mode == MODE_DENSE) {
+    if (P.mode == MODE_DENSE) {
       const int64_t gi = (int64_t)blk.rb * BM + row;
 #pragma unroll
       for (int c = 0; c < EPI_COLS / 32; ++c) {
@@ -1098,11 +849,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_heads(const __grid_constant__
 }
 
 // ------------------------------------------------------------- host side
+}  // namespace
+
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_encode_once;
 
 bool get_encode() {
-  std::call_once(g_encode_once, [] {
+  static std::once_flag once;
+  std::call_once(once, [] {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
@@ -1112,6 +865,8 @@ bool get_encode() {
   });
   return g_encode != nullptr;
 }
+
+namespace {
 
 // 2-D fp32 row-major matrix (rows x cols, row stride ld elements), box of
 // 32 columns (128 bytes, one swizzle row) by box_rows rows, 128-byte swizzle.
@@ -1146,21 +901,6 @@ bool make_map_pair(CUtensorMap* map, const float* hi, const float* lo, int64_t r
   return r == CUDA_SUCCESS;
 }
 
-// 2-D bf16 row-major matrix (rows x cols, row stride ld elements), box of 64
-// columns (128 bytes, one swizzle row) by box_rows rows, 128-byte swizzle.
-bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld,
-                   int box_rows) {
-  if (!get_encode() || (ld * 2) % 16) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)(ld * 2)};
-  cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1u, 1u};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)base, dims, strides,
-                        box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 bool g_attr_done = false;
 std::mutex g_attr_mu;
 
@@ -1170,12 +910,6 @@ cudaError_t ensure_attr() {
   cudaError_t e =
       cudaFuncSetAttribute(k_tc_band<V_BAND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            SMEM_BYTES);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_band<V_GRAM_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             SMEM_BYTES);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_band<V_GRAM_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             SMEM_BYTES);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_tc_band<V_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              PAIR_SMEM_BYTES);
@@ -1214,109 +948,6 @@ __global__ void k_split(const float* src, int64_t count, float* hi, float* lo) {
   const float v = src[i], h = tf32_hi(v);
   hi[i] = h;
   lo[i] = v - h;
-}
-
-// Gram operands: samples t0 .. t0 + kc of X (k x d, row stride ldx, fp32 or
-// bf16) transposed into the K-major planes T = X^T (dp x kc, zeros past k and
-// d), split as hi + lo; with weights, also WT = (diag(w) X)^T, the product
-// w_t x_ti rounded once to fp32 before the split.  32 x 32 tiles through
-// shared memory: coalesced reads along features, writes along samples.
-__global__ void k_gram_split(const void* X, int xdt, int k, int d, int64_t ldx, int t0, int kc,
-                             const float* w, float* Th, float* Tl, float* Wh, float* Wl) {
-  __shared__ float tile[32][33];
-  __shared__ float wt[32];
-  const int tx = threadIdx.x, ty = threadIdx.y;     // 32 x 8
-  const int tb = blockIdx.x * 32, ib = blockIdx.y * 32;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int t = t0 + tb + ty + 8 * r, i = ib + tx;
-    float v = 0.f;
-    if (t < k && i < d) {
-      const int64_t o = (int64_t)t * ldx + i;
-      v = xdt == BAKRON_BF16 ? __bfloat162float(((const __nv_bfloat16*)X)[o])
-                             : ((const float*)X)[o];
-    }
-    tile[ty + 8 * r][tx] = v;
-  }
-  if (w && ty == 0) wt[tx] = (t0 + tb + tx < k) ? w[t0 + tb + tx] : 0.f;
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = ib + ty + 8 * r, tc = tb + tx;
-    const int64_t o = (int64_t)i * kc + tc;
-    const float v = tile[tx][ty + 8 * r], h = tf32_hi(v);
-    Th[o] = h;
-    Tl[o] = v - h;
-    if (w) {
-      const float u = wt[tx] * v, uh = tf32_hi(u);
-      Wh[o] = uh;
-      Wl[o] = u - uh;
-    }
-  }
-}
-
-// bf16 samples t0 .. t0 + kc of X (k x d, row stride ldx) transposed into
-// the K-major bf16 plane T = X^T (dp x kc, zeros past k and d): the operand of
-// the kind::f16 Gram, exact (no split).  64 x 64 tiles through shared memory,
-// 16-byte vectors both ways: a load is 8 features of one sample (when X and
-// ldx allow 16-byte alignment and the 8 lie inside d; else element by
-// element), a store 8 samples of one feature (always whole: dp and kc are
-// multiples of 64).  A warp reads 4 rows of 128 bytes and stores 32 rows'
-// 16-byte pieces; its shared-memory gathers read one 64-byte row segment.
-constexpr int TR_TILE = 64, TR_LD = 72;   // row stride 144 B: 16-byte aligned rows
-
-__global__ void __launch_bounds__(256)
-    k_gram_transpose_bf16(const __nv_bfloat16* X, int k, int d, int64_t ldx, int t0, int kc,
-                          int vec_ok, __nv_bfloat16* T) {
-  __shared__ __align__(16) __nv_bfloat16 tile[TR_TILE][TR_LD];
-  const int tb = blockIdx.x * TR_TILE, ib = blockIdx.y * TR_TILE;
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int c = threadIdx.x + 256 * r;          // 512 chunks of 8 features
-    const int tr = c >> 3, i0 = ib + 8 * (c & 7);
-    const int t = t0 + tb + tr;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (t < k) {
-      const __nv_bfloat16* src = X + (int64_t)t * ldx + i0;
-      if (vec_ok && i0 + 8 <= d) {
-        v = *reinterpret_cast<const uint4*>(src);
-      } else {
-        __align__(16) __nv_bfloat16 e[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) e[j] = (i0 + j < d) ? src[j] : __float2bfloat16(0.f);
-        v = *reinterpret_cast<const uint4*>(e);
-      }
-    }
-    *reinterpret_cast<uint4*>(&tile[tr][8 * (c & 7)]) = v;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int c = threadIdx.x + 256 * r;          // 512 chunks of 8 samples
-    const int ir = c & 63, tc = c >> 6;
-    __align__(16) __nv_bfloat16 e[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) e[j] = tile[8 * tc + j][ir];
-    *reinterpret_cast<uint4*>(T + (int64_t)(ib + ir) * kc + tb + 8 * tc) =
-        *reinterpret_cast<const uint4*>(e);
-  }
-}
-
-// |y_t|^2 per row (warp per row, fp32, lane-strided partial sums then a
-// butterfly): the one-step Shampoo weight tr(b_t^T b_t) of a vector sample.
-__global__ void k_sqnorms(const void* Y, int ydt, int k, int d, int64_t ldy, float* out) {
-  const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= k) return;
-  float acc = 0.f;
-  for (int j = lane; j < d; j += 32) {
-    const int64_t o = row * ldy + j;
-    const float v = ydt == BAKRON_BF16 ? __bfloat162float(((const __nv_bfloat16*)Y)[o])
-                                       : ((const float*)Y)[o];
-    acc = fmaf(v, v, acc);
-  }
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) out[row] = acc;
 }
 
 }  // namespace
@@ -1541,103 +1172,4 @@ extern "C" int bakron_diag_gemm_tf32x3(const float* A, const float* B, float* C,
   }
   BK_CUDA_OK(cudaGetLastError());
   return bakron_read_status(workspace, stream);
-}
-
-// ------------------------------------------------------------ Gram matrices
-namespace {
-constexpr int GRAM_MAX_D = 1 << 16;
-}  // namespace
-
-extern "C" size_t bakron_gram_workspace_bytes(int d, int k_chunk, int weighted) {
-  if (d < 1 || d > GRAM_MAX_D || k_chunk < 1) return 0;
-  const int64_t dp = round_up(d, BM), kc = round_up(k_chunk, BK);
-  return 256 + (size_t)(weighted ? 4 : 2) * (size_t)dp * (size_t)kc * 4;
-}
-
-extern "C" int bakron_gram(const void* X, int xdtype, int k, int d, int64_t ldx, const float* w,
-                           float alpha, float beta, float* G, int64_t ldg, void* workspace,
-                           size_t workspace_bytes, int sync, void* stream) {
-  if (!X || !G || !workspace || k < 1 || d < 1 || d > GRAM_MAX_D || ldx < d || ldg < d)
-    return BAKRON_ERR_INVALID_ARG;
-  if (xdtype != BAKRON_F32 && xdtype != BAKRON_BF16) return BAKRON_ERR_INVALID_ARG;
-  const int64_t dp = round_up(d, BM);
-  // bf16 samples without weights: one exact bf16 plane, kind::f16 MMAs, K = 64
-  // per ring slot; otherwise tf32 hi/lo planes (two, or four with weights)
-  const bool bf16_ops = xdtype == BAKRON_BF16 && !w;
-  const int64_t kq = bf16_ops ? 2 * BK : BK;              // chunk granularity
-  const size_t per_sample = bf16_ops ? (size_t)dp * 2 : (size_t)(w ? 4 : 2) * dp * 4;
-  if (workspace_bytes < 256) return BAKRON_ERR_WORKSPACE;
-  int64_t kc = (int64_t)((workspace_bytes - 256) / per_sample) / kq * kq;
-  kc = std::min<int64_t>(kc, round_up(k, kq));
-  kc = std::min<int64_t>(kc, (int64_t)1 << 30);
-  if (kc < kq) return BAKRON_ERR_WORKSPACE;
-  BK_CUDA_OK(ensure_attr());
-  cudaStream_t s = (cudaStream_t)stream;
-  char* ws = (char*)workspace;
-  int* status = (int*)ws;
-  float* Th = (float*)(ws + 256);
-  float* Tl = Th + dp * kc;
-  float* Wh = w ? Tl + dp * kc : nullptr;
-  float* Wl = w ? Wh + dp * kc : nullptr;
-  BK_CUDA_OK(cudaMemsetAsync(status, 0, 256, s));
-  const int nb = (int)(dp / BM);
-  const unsigned ntri = (unsigned)((int64_t)nb * (nb + 1) / 2);
-  const long long spin = spin_cycles_from_env();
-  for (int64_t t0 = 0; t0 < k; t0 += kc) {
-    const int64_t kcl = std::min<int64_t>(kc, round_up(k - t0, kq));   // this chunk's K
-    dim3 sg((unsigned)(kcl / 32), (unsigned)(dp / 32));
-    CUtensorMap mA2, mB2;
-    if (bf16_ops) {
-      __nv_bfloat16* Tb = (__nv_bfloat16*)(ws + 256);
-      const int vec_ok = ((uintptr_t)X % 16 == 0 && ldx % 8 == 0) ? 1 : 0;
-      dim3 tg((unsigned)(kcl / TR_TILE), (unsigned)(dp / TR_TILE));
-      k_gram_transpose_bf16<<<tg, 256, 0, s>>>((const __nv_bfloat16*)X, k, d, ldx, (int)t0,
-                                               (int)kc, vec_ok, Tb);
-      BK_CUDA_OK(cudaGetLastError());
-      if (!make_map_bf16(&mA2, Tb, dp, kcl, kc, BM) || !make_map_bf16(&mB2, Tb, dp, kcl, kc, BN))
-        return BAKRON_ERR_CUDA;
-    } else {
-      k_gram_split<<<sg, dim3(32, 8), 0, s>>>(X, xdtype, k, d, ldx, (int)t0, (int)kc, w, Th, Tl,
-                                              Wh, Wl);
-      BK_CUDA_OK(cudaGetLastError());
-      const float* ah = w ? Wh : Th;
-      const float* al = w ? Wl : Tl;
-      if (!make_map_pair(&mA2, ah, al, dp, kcl, kc, BM) ||
-          !make_map_pair(&mB2, Th, Tl, dp, kcl, kc, BN))
-        return BAKRON_ERR_CUDA;
-    }
-    TcParams P{};
-    P.mode = MODE_GRAM;
-    P.K = (int)kcl;
-    P.out_hi = G;
-    P.ldo = ldg;
-    P.status = status;
-    P.spin_cycles = spin;
-    P.alpha = alpha;
-    P.beta = t0 == 0 ? beta : 1.f;
-    P.dreal = d;
-    P.b_exact = xdtype == BAKRON_BF16;              // bf16 is exact in tf32: lo plane zero
-    P.a_exact = xdtype == BAKRON_BF16 && !w;
-    // bf16: K counted in 128-byte rows of 64; exact products, GRAM_KGROUP
-    // slots (256 samples) per accumulator hand-over
-    if (bf16_ops) {
-      P.K = (int)(kcl / 2);
-      k_tc_band<V_GRAM_BF16><<<ntri, THREADS, SMEM_BYTES, s>>>(mA2, mB2, mB2, mB2, mB2, mB2, P);
-    } else {
-      k_tc_band<V_GRAM_TF32><<<ntri, THREADS, SMEM_BYTES, s>>>(mA2, mB2, mB2, mB2, mB2, mB2, P);
-    }
-    BK_CUDA_OK(cudaGetLastError());
-  }
-  if (!sync) return BAKRON_OK;
-  return bakron_read_status(workspace, stream);
-}
-
-extern "C" int bakron_sample_sqnorms(const void* Y, int ydtype, int k, int d, int64_t ldy,
-                                     float* out, void* stream) {
-  if (!Y || !out || k < 1 || d < 1 || ldy < d) return BAKRON_ERR_INVALID_ARG;
-  if (ydtype != BAKRON_F32 && ydtype != BAKRON_BF16) return BAKRON_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  k_sqnorms<<<(unsigned)(((int64_t)k * 32 + 255) / 256), 256, 0, s>>>(Y, ydtype, k, d, ldy, out);
-  BK_CUDA_OK(cudaGetLastError());
-  return BAKRON_OK;
 }
