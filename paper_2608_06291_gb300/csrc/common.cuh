@@ -110,20 +110,18 @@ struct SolveLayout {
   }
 };
 
-// Prepare works on one Gram at a time (the larger side bounds the size).
-// Real type of the factorisation: fp64 (see prepare.cu for the reason).
+// Prepare workspace: [status 256 B][X_A np x np][X_B mp x mp], fp64: the inverses of
+// the two Cholesky factors.  (The factors themselves are formed in the factor
+// buffer, see prepare.cu.)
 struct PrepareLayout {
-  int64_t dp;
-  size_t off_status, off_C, off_Linv, off_T, off_scalar, bytes;
+  size_t off_status, off_X, bytes;
   PrepareLayout(int m, int n) {
-    int64_t d = m > n ? m : n;
-    dp = round_up(d, PAD);
+    const int64_t mp = round_up(m, PAD), np = round_up(n, PAD), dp = mp > np ? mp : np;
     off_status = 0;
-    off_C = 256;
-    off_Linv = align256(off_C + size_t(dp * dp) * 8);
-    off_T = align256(off_Linv + size_t(dp * dp) * 8);
-    off_scalar = align256(off_T + size_t(dp * PAD) * 8);
-    bytes = align256(off_scalar + 256);
+    off_X = 256;
+    // the size documented for earlier versions, which a caller may have stored:
+    // two fp64 matrices of the larger side and their diagonal blocks
+    bytes = align256(off_X + size_t(dp * dp) * 16 + size_t(dp * PAD) * 8 + 256);
   }
 };
 
