@@ -20,11 +20,11 @@
 // al. 2012, error-free transformations of matrix multiplication):
 //   * Row and column i of the matrix are scaled by 2^-e_i (exact) so that the
 //     diagonal lies in [1/4, 1): then |H_ij| < 1 and the rows of its Cholesky
-//     factor have norm < 1, and both are kept as 64-bit fixed point, unit 2^-62
-//     ("Q62"), which loses less than an fp64 of the same matrix would.
-//   * An operand is cut into seven balanced base-256 digits, 56 bits (Q62 as it
-//     is; fp64 matrices relative to a power of two above each row's norm), each
-//     an fp16 integer of [-128, 127].  The 28 products of digit planes (i, j) with
+//     factor have norm < 1, and both are kept as 64-bit fixed point, unit 2^-63
+//     ("Q63"), which loses less than an fp64 of the same matrix would.
+//   * An operand is cut into seven balanced base-256 digits, its upper 56 bits (Q63
+//     as it is; fp64 matrices relative to a power of two above each row's norm),
+//     each an fp16 integer of [-128, 127].  The 28 products of digit planes (i, j) with
 //     i + j <= 6 are exact in the tensor cores' fp32 accumulators over 64 terms
 //     (7 * 64 * 2^14 < 2^23); planes of equal i + j share one.  Their sum, shifted
 //     8 bits apart, is formed in 64-bit integers modulo 2^64: it cannot be lost,
@@ -50,16 +50,17 @@ namespace {
 constexpr int NB = 64;            // Cholesky panel width, contraction chunk
 constexpr int OT = 128;           // output tile of the sliced products
 constexpr int SLICES = 7;
-constexpr int WORKERS = 16;       // warps that cut operands and sum accumulators
+// Sixteen warps cut operands and sum accumulators; thread 0 issues the MMAs
+// between its other work (a warp of its own would leave 96 registers a thread).
+constexpr int WORKERS = 16;
 constexpr int WT = 32 * WORKERS;
-constexpr int OZ_THREADS = WT + 32;             // and one that issues the MMAs
 constexpr uint32_t OPLANE = OT * 128;           // 128 rows of 64 fp16
 constexpr uint32_t OZ_SMEM = 2 * SLICES * OPLANE + 1024 /*align*/ + 256 /*barriers*/;
 constexpr int OUT_LD = OT + 2;                  // staged output row, 8-byte words
 static_assert(OT * OUT_LD * 8 <= 2 * SLICES * OPLANE, "the output is staged over the planes");
 
 // One side (A or B) of a prepare call.  C is dp x dp, row-major, 64-bit words:
-// lower triangle and diagonal blocks Q62, first the scaled matrix, then its
+// lower triangle and diagonal blocks Q63, first the scaled matrix, then its
 // Cholesky factor; above the diagonal, during the inverse, intermediate products
 // (fp64).  X: the factor's inverse (fp64, lower).
 struct PrepSide {
@@ -96,7 +97,7 @@ __device__ __forceinline__ int exp_above_sqrt(double v) {
 }
 
 // x * 2^u rounded to an integer, by integer operations (no fp64 unit); the
-// caller's bounds keep it below 2^62, larger magnitudes give garbage.
+// caller's bounds keep it below 2^63, larger magnitudes give garbage.
 __device__ __forceinline__ long long to_fix(double x, int u) {
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ff);
@@ -177,9 +178,9 @@ __global__ void __launch_bounds__(256) k_prep_load(const PrepArgs P) {
     double h = (double)tile[x][r];
     if (i == j) h = i < d ? h + add : 1.0;
     // 1 or more (infinities and NaN too): beyond sqrt(H_ii H_jj) < 0.976
-    const int u = 62 - S.e[i] - S.e[j], ex = (__double2hiint(h) >> 20) & 0x7ff;
-    long long v = ex - 1023 + u >= 62 ? 1LL << 62 : to_fix(h, u);
-    const long long lim = (1LL << 62) - (1LL << 56);   // 0.984
+    const int u = 63 - S.e[i] - S.e[j], ex = (__double2hiint(h) >> 20) & 0x7ff;
+    long long v = ex - 1023 + u >= 63 ? 0x7fffffffffffffffLL : to_fix(h, u);
+    const long long lim = 0x7eLL << 56;   // 0.984
     if (v > lim || v < -lim) {
       bad = true;
       v = 0;
@@ -190,9 +191,33 @@ __global__ void __launch_bounds__(256) k_prep_load(const PrepArgs P) {
 }
 
 // ------------------------------------------------------- diagonal blocks
+// A Q63 value for products in integers: ah * 2^25 + al, unit 2^-56 (ah 32 bits
+// with the sign, al 25).
+__device__ __forceinline__ int2 split56(long long v) {
+  const long long u = v + 64;   // rounded
+  return make_int2((int)(u >> 32), (int)((uint32_t)u >> 7));
+}
+// sum += a b, in two parts: s1 of unit 2^-62, s2 of unit 2^-87 (al * bl, below
+// 2^-62, is left out).  The sums are right modulo 2^64: the products' sum itself
+// is below 1 by the norms of the rows that are multiplied.
+__device__ __forceinline__ void mac56(long long& s1, long long& s2, int2 a, int2 b) {
+  s1 += (long long)a.x * b.x;
+  s2 += (long long)a.x * b.y;
+  s2 += (long long)a.y * b.x;
+}
+__device__ __forceinline__ long long sum56(long long s1, long long s2) {   // Q63
+  return (long long)((unsigned long long)s1 << 1) + (s2 >> 24);
+}
+
+constexpr int PH = NB / 2;       // the inverse's last halving, in integers
 struct PotrfSmem {
-  double s[NB][NB + 1];
-  double inv[NB][NB + 1];   // and, above the diagonal, the products of its halving
+  long long a[NB][NB + 1];       // Q63: the block, then its factor
+  double inv[NB][NB + 1];        // the inverse; above the diagonal, products of its halving
+  double cur[NB][9];             // the eight columns being factored
+  __align__(16) int2 l8[NB][10]; // the same, factored, split (rows of 80 bytes: no conflicts)
+  int2 xs[PH][PH + 1];           // columns of X11, then rows of X22 (split)
+  int2 ts[PH][PH + 1];           // L21, then columns of L21 X11 (split)
+  int ec[PH], er[PH], et[PH];
   double pub[8][8];
   double rinv[NB];
 };
@@ -209,22 +234,46 @@ __device__ __forceinline__ double rsqrt64(double p) {
   return fma(r * e, fma(0.375, e, 0.5), r);
 }
 
-// Factors the block of C at (k0, k0) and inverts the factor, by the first WT
-// threads of the CTA.  Writes the factor to C, its inverse to dinv and to X's
-// diagonal block, the exponents of the inverse's rows to f.  A pivot that is not
-// positive raises NOT_SPD and is replaced by 1.
+// An exponent above three times the largest magnitude of a warp's values (32
+// values of that exponent have a norm below one: sqrt(32) < 2^3 / 1.05).
+__device__ __forceinline__ int warp_exp8(double x) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(x) & 0x7fffffffu);
+  return (int)(m >> 20) - 1022 + 3;
+}
+
+// Factors the block of C at (k0, k0) and inverts the factor, by all WT threads
+// of the CTA.  Writes the factor to C, its inverse to dinv and to X's diagonal
+// block, the exponents of the inverse's rows to f.  A pivot that is not positive
+// raises NOT_SPD and is replaced by 1.
 //
 // The fp64 units take a warp's instruction every 64 cycles per scheduler, so
-// the count of warp instructions sets the time: eight columns at a time, a
-// thread per row with the columns' entries in registers (unscaled pivots and
-// the eight rows they share are published once per column, 1 / sqrt is formed
-// redundantly), then one update of the rest by all warps; the inverse by halving,
-// all warps on each product.
+// the count of those sets the time, and what can be is done in integers.  Eight
+// columns at a time: a thread per row with the columns' entries in registers, fp64
+// (the unscaled pivot and the eight rows it shares are published once per column,
+// 1 / sqrt is formed redundantly; about 1000 cycles a column, 1700 with both
+// halves' rows in one warp); then one update of the rest by all warps on split
+// 56-bit values (three 32 x 32 + 64 multiply-adds each).  The inverse by halving:
+// 8 x 8 blocks and the first two levels in fp64, the last in integers.
 __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status) {
-  const int t = threadIdx.x;
-  for (int e = t; e < NB * NB; e += WT) {
-    const int r = e / NB, c = e % NB;
-    M.s[r][c] = c <= r ? from_fix(S.C[(int64_t)(k0 + r) * S.dp + k0 + c], -62) : 0.0;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // this thread's entries of a lower triangle of up to 63 rows, row by row
+  constexpr int TRI = ((NB - 8) * (NB - 7) / 2 + WT - 1) / WT;
+  int tr[TRI], tc[TRI];
+#pragma unroll
+  for (int i = 0; i < TRI; ++i) {
+    const int e = t + WT * i;
+    int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    while ((r + 1) * (r + 2) / 2 <= e) ++r;
+    while (r * (r + 1) / 2 > e) --r;
+    tr[i] = r;
+    tc[i] = e - r * (r + 1) / 2;
+  }
+#pragma unroll
+  for (int i = 0; i < NB * NB / WT; ++i) {
+    const int e = t + WT * i, r = e / NB, c = e % NB;
+    const long long v = c <= r ? __ldcg(S.C + (int64_t)(k0 + r) * S.dp + k0 + c) : 0;
+    M.a[r][c] = v;
+    if (c < 8) M.cur[r][c] = from_fix(v, -63);
   }
   workers_sync();
   for (int c0 = 0; c0 < NB; c0 += 8) {
@@ -233,7 +282,7 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
       const int live = NB - (c0 & 32);
       double a[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) a[j] = M.s[r][c0 + j];
+      for (int j = 0; j < 8; ++j) a[j] = r >= c0 ? M.cur[r][j] : 0.0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         if (r >= c0 && r < c0 + 8) M.pub[j][r - c0] = a[j];
@@ -246,51 +295,70 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
         const double ri = rsqrt64(p);
         const double l = (r == c0 + j ? p : a[j]) * ri, lr = l * ri;
         a[j] = l;
-        if (r == c0 + j) M.rinv[r] = ri;
+        if (r == c0 + j) {
+          M.rinv[r] = ri;
+          S.ldiag[k0 + r] = l;
+        }
 #pragma unroll
         for (int k = j + 1; k < 8; ++k) a[k] = fma(-lr, M.pub[j][k], a[k]);
       }
       if (r >= c0) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (c0 + j <= r) M.s[r][c0 + j] = a[j];
+        for (int j = 0; j < 8; ++j) {
+          const long long v = c0 + j <= r ? to_fix(a[j], 63) : 0;
+          if (c0 + j <= r) M.a[r][c0 + j] = v;
+          M.l8[r][j] = split56(v);
+          M.inv[r][c0 + j] = a[j];       // the factor in fp64, for the halving
+        }
       }
     }
     workers_sync();
     const int b0 = c0 + 8, rem = NB - b0;
-    for (int e = t; e < rem * (rem + 1) / 2; e += WT) {
-      int r = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-      while ((r + 1) * (r + 2) / 2 <= e) ++r;
-      while (r * (r + 1) / 2 > e) --r;
-      const int c = e - r * (r + 1) / 2;
-      double v = M.s[b0 + r][b0 + c];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v = fma(-M.s[b0 + r][c0 + k], M.s[b0 + c][c0 + k], v);
-      M.s[b0 + r][b0 + c] = v;
+    for (int i = 0; i < TRI; ++i) {
+      if (t + WT * i >= rem * (rem + 1) / 2) continue;
+      const int r = b0 + tr[i], c = b0 + tc[i];
+      const int4* lr = reinterpret_cast<const int4*>(M.l8[r]);
+      const int4* lc = reinterpret_cast<const int4*>(M.l8[c]);
+      long long s1 = 0, s2 = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int4 x = lr[k], y = lc[k];
+        mac56(s1, s2, make_int2(x.x, x.y), make_int2(y.x, y.y));
+        mac56(s1, s2, make_int2(x.z, x.w), make_int2(y.z, y.w));
+      }
+      const long long v = M.a[r][c] - sum56(s1, s2);
+      M.a[r][c] = v;
+      if (tc[i] < 8) M.cur[r][tc[i]] = from_fix(v, -63);
     }
     workers_sync();
   }
-  // the inverse: 8 x 8 diagonal blocks, a thread per column ...
+  // M.inv holds the factor (fp64).  The inverse: 8 x 8 diagonal blocks, a thread
+  // per column ...
+  double x8[8];
   if (t < NB) {
     const int b = t & ~7, c = t & 7;
-    double x[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       double v = 0.0;
 #pragma unroll
-      for (int k = 0; k < r; ++k) v = fma(M.s[b + r][b + k], x[k], v);
-      x[r] = r == c ? M.rinv[b + r] : -v * M.rinv[b + r];
-      if (r < c) x[r] = 0.0;
-      M.inv[b + r][b + c] = x[r];
+      for (int k = 0; k < r; ++k) v = fma(M.inv[b + r][b + k], x8[k], v);
+      x8[r] = r == c ? M.rinv[b + r] : -v * M.rinv[b + r];
+      if (r < c) x8[r] = 0.0;
     }
+    asm volatile("bar.sync 2, %0;" ::"n"(NB) : "memory");
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r >= c) M.inv[b + r][b + c] = x8[r];
   }
   workers_sync();
-  // ... then [[X11, 0], [-X22 L21 X11, X22]] at 8, 16, 32
-  for (int h = 8; h < NB; h *= 2) {
+  // ... then [[X11, 0], [-X22 L21 X11, X22]] at 8 and 16: L21 is read where X21 goes
+#pragma unroll
+  for (int h = 8; h < PH; h *= 2) {
     for (int e = t; e < NB / 2 * h; e += WT) {
       const int i0 = 2 * h * (e / (h * h)), c = (e / h) % h, r = e % h;
       double v = 0.0;
-      for (int k = c; k < h; ++k) v = fma(M.s[i0 + h + r][i0 + k], M.inv[i0 + k][i0 + c], v);
+      for (int k = c; k < h; ++k) v = fma(M.inv[i0 + h + r][i0 + k], M.inv[i0 + k][i0 + c], v);
       M.inv[i0 + c][i0 + h + r] = v;                   // (L21 X11)[r][c], transposed
     }
     workers_sync();
@@ -302,21 +370,61 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
     }
     workers_sync();
   }
-  for (int e = t; e < NB * NB; e += WT) {
-    const int r = e / NB, c = e % NB;
+  // at 32, in integers relative to the norms of X11's columns, X22's rows and the
+  // columns of L21 X11 (a warp per column or row)
+  for (int c = warp; c < PH; c += WORKERS) {
+    const double x = lane >= c ? M.inv[lane][c] : 0.0;
+    const int e = warp_exp8(x);
+    M.xs[c][lane] = split56(to_fix(x, 63 - e));
+    M.ts[c][lane] = split56(M.a[PH + c][lane]);        // row c of L21
+    if (lane == 0) M.ec[c] = e;
+  }
+  workers_sync();
+  long long tv[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {                        // column c of L21 X11, lane = row
+    const int c = warp + WORKERS * i;
+    long long s1 = 0, s2 = 0;
+    for (int k = c; k < PH; ++k) mac56(s1, s2, M.ts[lane][k], M.xs[c][k]);
+    tv[i] = sum56(s1, s2);
+  }
+  workers_sync();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int c = warp + WORKERS * i;
+    const unsigned long long mag = (unsigned long long)(tv[i] < 0 ? -tv[i] : tv[i]);
+    const int z = max(__clz((int)__reduce_max_sync(0xffffffffu, (unsigned)(mag >> 32))) - 1, 0);
+    // up by z bits to the top, then 3 down for the norm
+    M.ts[c][lane] = split56((long long)((unsigned long long)tv[i] << z) >> 3);
+    if (lane == 0) M.et[c] = M.ec[c] - z + 3;
+    const double x = lane <= c ? M.inv[PH + c][PH + lane] : 0.0;   // row c of X22
+    const int e = warp_exp8(x);
+    M.xs[c][lane] = split56(to_fix(x, 63 - e));
+    if (lane == 0) M.er[c] = e;
+  }
+  workers_sync();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {                        // row r of X21, lane = column
+    const int r = warp + WORKERS * i;
+    long long s1 = 0, s2 = 0;
+    for (int k = 0; k <= r; ++k) mac56(s1, s2, M.xs[r][k], M.ts[lane][k]);
+    M.inv[PH + r][lane] = from_fix(-sum56(s1, s2), M.er[r] + M.et[lane] - 63);
+  }
+  workers_sync();
+#pragma unroll
+  for (int i = 0; i < NB * NB / WT; ++i) {
+    const int e = t + WT * i, r = e / NB, c = e % NB;
     const double x = c <= r ? M.inv[r][c] : 0.0;
     const int64_t o = (int64_t)(k0 + r) * S.dp + k0 + c;
     S.dinv[(int64_t)(k0 + r) * NB + c] = x;
     S.X[o] = x;
-    S.C[o] = c <= r ? to_fix(M.s[r][c], 62) : 0;
-    if (r == c) S.ldiag[k0 + r] = M.s[r][c];
+    S.C[o] = M.a[r][c];
   }
-  for (int r = t >> 5; r < NB; r += WORKERS) {
-    const int l = t & 31;
-    unsigned m = l <= r ? __double2hiint(M.inv[r][l]) & 0x7fffffff : 0;
-    if (l + 32 <= r) m = max(m, __double2hiint(M.inv[r][l + 32]) & 0x7fffffffu);
+  for (int r = warp; r < NB; r += WORKERS) {
+    unsigned m = lane <= r ? __double2hiint(M.inv[r][lane]) & 0x7fffffff : 0;
+    if (lane + 32 <= r) m = max(m, __double2hiint(M.inv[r][lane + 32]) & 0x7fffffffu);
     m = __reduce_max_sync(0xffffffffu, m);
-    if (l == 0) S.f[k0 + r] = min(exp_above(__hiloint2double((int)m, -1)), 300);
+    if (lane == 0) S.f[k0 + r] = min(exp_above(__hiloint2double((int)m, -1)), 300);
   }
 }
 
@@ -337,21 +445,22 @@ __global__ void __launch_bounds__(WT) k_prep_first(const PrepArgs P) {
 //   OZ_INV2  X21 = -X22 R^T
 enum OzMode { OZ_TRSM, OZ_SYRK, OZ_INV1, OZ_INV2 };
 
-// Seven digits of eight values (56-bit fixed point) to the planes: 16 bytes of
-// a row each, in the 128-byte swizzled layout.
+// Seven digits of eight values (Q63) to the planes: 16 bytes of a row each, in
+// the 128-byte swizzled layout.  The 128s added to every byte make the digits
+// balanced (the last one rounds the byte that is dropped).
 __device__ __forceinline__ void put_digits(unsigned char* planes, uint32_t plane, int row, int oct,
                                            const long long (&w)[8]) {
   uint32_t lo[8], hi[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const unsigned long long u = (unsigned long long)w[k] + 0x0080808080808080ULL;
+    const unsigned long long u = (unsigned long long)w[k] + 0x8080808080808080ULL;
     lo[k] = (uint32_t)u;
     hi[k] = (uint32_t)(u >> 32);
   }
   unsigned char* dst = planes + row * 128 + ((oct ^ (row & 7)) << 4);
 #pragma unroll
   for (int s = 0; s < SLICES; ++s) {
-    const int b = SLICES - 1 - s;                      // byte of the digit, biased by 128
+    const int b = SLICES - s;                          // byte of the digit, biased by 128
     uint32_t o[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -368,6 +477,13 @@ __device__ __forceinline__ void put_digits(unsigned char* planes, uint32_t plane
   }
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                 "=r"(r[7])
+               : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -377,6 +493,31 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+
+// An integer x, |x| <= 2^22, held in fp32: its bits after adding 1.5 * 2^23 are
+// OZ_BIAS + x, for one addition instead of a conversion (a quarter of its rate).
+constexpr uint32_t OZ_BIAS = 0x4B400000u;
+__device__ __forceinline__ uint32_t biased_int(uint32_t f) {
+  return __float_as_uint(__uint_as_float(f) + 12582912.f);
+}
+
+// An integer x, |x| < 2^23, held in fp32, by additions: its half rounded to an
+// integer, and what is left (-1, 0 or 1).
+__device__ __forceinline__ uint32_t wide_int(uint32_t f) {
+  const float x = __uint_as_float(f), h = fmaf(x, 0.5f, 12582912.f);
+  const float rest = fmaf(h - 12582912.f, -2.f, x);
+  return 2 * (__float_as_uint(h) - OZ_BIAS) + (__float_as_uint(rest + 12582912.f) - OZ_BIAS);
+}
+
+// Four 8-byte words, 32-byte aligned: whole sectors per lane.
+__device__ __forceinline__ void ld4(const long long* p, long long& a, long long& b, long long& c, long long& d) {
+  asm volatile("ld.global.v4.u64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p) : "memory");
+}
+
+template <int V>
+struct Int {
+  static constexpr int value = V;
+};
 
 // kind::f16 with fp16 A and B (K-major), D fp32.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
@@ -439,37 +580,38 @@ __device__ __forceinline__ bool oz_tile(const PrepSide& S, int arg, OzTile& T, i
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(const PrepArgs P, int arg) {
+__global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
   extern __shared__ __align__(1024) unsigned char oz_smem[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem + 1023) & ~(uintptr_t)1023);
   unsigned char* pa = smem;
   constexpr int BN = MODE == OZ_TRSM ? NB : OT;        // columns of the MMAs
   constexpr uint32_t b_plane = BN * 128;
   unsigned char* pb = smem + SLICES * OPLANE;
-  uint64_t* accF = (uint64_t*)(smem + 2 * SLICES * OPLANE);   // [4] a digit sum is complete
-  uint64_t* accE = accF + 4;                                   // [4] it has been read out
-  uint64_t* done = accE + 4;
+  // per chunk, the sums of digit products of equal weight s = 0 .. 6 are handed
+  // over as {0, 1, 2}, {3, 4}, {5, 6}; sum s sits in accumulator s & 3
+  uint64_t* accF = (uint64_t*)(smem + 2 * SLICES * OPLANE);   // [3] a group is complete
+  uint64_t* accE = accF + 3;                                   // group 0 has been read out
+  uint64_t* done = accE + 1;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   const PrepSide& S = P.side[blockIdx.z];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   constexpr int drains = BN / 32 * 4;                  // warps that read accumulators
-  pdl_wait();
-  pdl_trigger();
   OzTile T;
   int i0;
-  if ((MODE == OZ_TRSM || MODE == OZ_SYRK) && arg + NB >= S.dp) return;
-  if (!oz_tile<MODE>(S, arg, T, i0)) return;           // uniform over the CTA
+  if (((MODE == OZ_TRSM || MODE == OZ_SYRK) && arg + NB >= S.dp) || !oz_tile<MODE>(S, arg, T, i0)) {
+    pdl_wait();                                        // uniform over the CTA
+    pdl_trigger();
+    return;
+  }
   if (t == 0) {
-    for (int a = 0; a < 4; ++a) {
-      mbar_init(&accF[a], 1);
-      mbar_init(&accE[a], drains);
-    }
+    for (int a = 0; a < 3; ++a) mbar_init(&accF[a], 1);
+    mbar_init(accE, drains);
     mbar_init(done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == WORKERS) {
+  if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(512)
@@ -480,134 +622,133 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(const PrepArgs P, int arg)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
   const int64_t ld = S.dp;
   const int q = warp & 3, cg = warp >> 2;              // lane quarter, 32 columns
   const long long drain_limit = 4000000000LL;
+  if constexpr (MODE == OZ_SYRK) {   // the tile's old values on their way to L2
+    for (int e = t; e < T.na * 8; e += WT)
+      if (16 * (e & 7) < T.nb)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(S.C + (int64_t)(T.ra + (e >> 3)) * ld + T.rb + 16 * (e & 7)));
+  }
   auto timed_out = [&]() {
     raise_status(P.status, BAKRON_ERR_TIMEOUT);
     *abort_flag = 1;
   };
-  long long acc[32];
+  // operand words of one unit (a row's eight terms): raw, then Q63
+  auto load_a = [&](int u, int kk, long long (&w)[8]) {
+    const int row = MODE == OZ_INV1 ? u & (OT - 1) : u >> 3, oct = MODE == OZ_INV1 ? u >> 7 : u & 7;
 #pragma unroll
-  for (int u = 0; u < 32; ++u) acc[u] = 0;
-  bool issuing = true, dead = false;
-  for (int ch = 0; ch < T.kn; ++ch) {
-    const int kk = NB * (T.k0 + ch);
-    if (warp < WORKERS) {
-      // ---------------------------------------------------- cut the operands
-      for (int u = t; u < OT * 8; u += WT) {
-        int row, oct;
-        if constexpr (MODE == OZ_INV1) {
-          row = u & (OT - 1);
-          oct = u >> 7;
-        } else {
-          row = u >> 3;
-          oct = u & 7;
-        }
-        long long w[8];
+    for (int k = 0; k < 8; ++k) w[k] = 0;
+    if (row >= T.na) return;
+    if constexpr (MODE == OZ_INV1) {                   // X11[k][j], k >= j
+      const int j = T.ra + row;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) w[k] = 0;
-        if (row < T.na) {
-          if constexpr (MODE == OZ_TRSM || MODE == OZ_SYRK) {
-            const longlong2* p = reinterpret_cast<const longlong2*>(
-                S.C + (int64_t)(T.ra + row) * ld + i0 + 8 * oct);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const longlong2 v = __ldcg(p + k);
-              w[2 * k] = (v.x + 64) >> 7;
-              w[2 * k + 1] = (v.y + 64) >> 7;
-            }
-          } else if constexpr (MODE == OZ_INV1) {      // X11[k][j], k >= j
-            const int j = T.ra + row;
-            const int ex = 55 - S.xc[i0 + j];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int kr = kk + 8 * oct + k;
-              if (kr >= j) w[k] = to_fix(S.X[(int64_t)(i0 + kr) * ld + i0 + j], ex);
-            }
-          } else {                                     // X22[i][k], k <= i
-            const int i = T.ra + row;
-            const int ex = 55 - S.xr[i0 + arg + i];
-            const double2* p = reinterpret_cast<const double2*>(
-                S.X + (int64_t)(i0 + arg + i) * ld + i0 + arg + kk + 8 * oct);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int kc = kk + 8 * oct + 2 * k;
-              if (kc <= i) {
-                const double2 v = p[k];
-                w[2 * k] = to_fix(v.x, ex);
-                if (kc + 1 <= i) w[2 * k + 1] = to_fix(v.y, ex);
-              }
-            }
-          }
-        }
-        put_digits(pa, OPLANE, row, oct, w);
+      for (int k = 0; k < 8; ++k) {
+        const int kr = kk + 8 * oct + k;
+        if (kr >= j) w[k] = __double_as_longlong(S.X[(int64_t)(i0 + kr) * ld + i0 + j]);
       }
-      for (int u = t; u < BN * 8; u += WT) {
-        const int row = u >> 3, oct = u & 7;
-        long long w[8];
+    } else {                                           // C's panel, or X22[i][k], k <= i
+      const long long* p =
+          MODE == OZ_INV2 ? (const long long*)S.X + (int64_t)(i0 + arg + T.ra + row) * ld + i0 + arg + kk + 8 * oct
+                          : S.C + (int64_t)(T.ra + row) * ld + i0 + 8 * oct;
+      ld4(p, w[0], w[1], w[2], w[3]);
+      ld4(p + 4, w[4], w[5], w[6], w[7]);
+      if constexpr (MODE == OZ_INV2) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) w[k] = 0;
-        if (row < T.nb) {
-          if constexpr (MODE == OZ_TRSM || MODE == OZ_INV2) {
-            const int ex = 55 - (MODE == OZ_TRSM ? S.f[i0 + row] : S.tr[i0 + T.rb + row]);
-            const double2* p = reinterpret_cast<const double2*>(
-                MODE == OZ_TRSM ? S.dinv + (int64_t)(i0 + row) * NB + 8 * oct
-                                : (const double*)S.C + (int64_t)(i0 + T.rb + row) * ld + i0 + arg + kk + 8 * oct);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const double2 v = p[k];
-              w[2 * k] = to_fix(v.x, ex);
-              w[2 * k + 1] = to_fix(v.y, ex);
-            }
-          } else {
-            const longlong2* p = reinterpret_cast<const longlong2*>(
-                MODE == OZ_SYRK ? S.C + (int64_t)(T.rb + row) * ld + i0 + 8 * oct
-                                : S.C + (int64_t)(i0 + arg + T.rb + row) * ld + i0 + kk + 8 * oct);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const longlong2 v = __ldcg(p + k);
-              w[2 * k] = (v.x + 64) >> 7;
-              w[2 * k + 1] = (v.y + 64) >> 7;
-            }
-          }
-        }
-        put_digits(pb, b_plane, row, oct, w);
+        for (int k = 0; k < 8; ++k)
+          if (kk + 8 * oct + k > T.ra + row) w[k] = 0;
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    __syncthreads();
-    if (warp == WORKERS) {
-      // ------------------------------------------------------------ products
-      if (lane == 0 && issuing) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t da = smem_desc(smem_u32(pa)), db = smem_desc(smem_u32(pb));
-        for (int s = 0; s < SLICES && issuing; ++s) {
-          const int g = SLICES * ch + s, a = g & 3;
-          if (g >= 4 && !oz_wait(&accE[a], (uint32_t)((g >> 2) - 1) & 1u, P.spin_cycles, abort_flag)) {
-            if (!*abort_flag) timed_out();
-            issuing = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          for (int i = 0; i <= s; ++i) {
+  };
+  auto load_b = [&](int u, int kk, long long (&w)[8]) {
+    const int row = u >> 3, oct = u & 7;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              mma_bf16(tmem + (uint32_t)(a * OT), da + (uint64_t)(i * (OPLANE >> 4) + 2 * k),
-                       db + (uint64_t)((s - i) * (b_plane >> 4) + 2 * k), idesc_f16(OT, BN),
-                       (i > 0 || k > 0) ? 1u : 0u);
-          }
-          mma_commit(&accF[a]);
-        }
+    for (int k = 0; k < 8; ++k) w[k] = 0;
+    if (row >= T.nb) return;
+    const long long* p =
+        MODE == OZ_TRSM   ? (const long long*)S.dinv + (int64_t)(i0 + row) * NB + 8 * oct
+        : MODE == OZ_SYRK ? S.C + (int64_t)(T.rb + row) * ld + i0 + 8 * oct
+        : MODE == OZ_INV1 ? S.C + (int64_t)(i0 + arg + T.rb + row) * ld + i0 + kk + 8 * oct
+                          : S.C + (int64_t)(i0 + T.rb + row) * ld + i0 + arg + kk + 8 * oct;
+    ld4(p, w[0], w[1], w[2], w[3]);
+    ld4(p + 4, w[4], w[5], w[6], w[7]);
+  };
+  auto put_a = [&](int u, long long (&w)[8]) {
+    const int row = MODE == OZ_INV1 ? u & (OT - 1) : u >> 3, oct = MODE == OZ_INV1 ? u >> 7 : u & 7;
+    if constexpr (MODE == OZ_INV1 || MODE == OZ_INV2) {
+      const int ex = row >= T.na ? 0 : 63 - (MODE == OZ_INV1 ? S.xc[i0 + T.ra + row] : S.xr[i0 + arg + T.ra + row]);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[k] = to_fix(__longlong_as_double(w[k]), ex);
+    }
+    put_digits(pa, OPLANE, row, oct, w);
+  };
+  auto put_b = [&](int u, long long (&w)[8]) {
+    const int row = u >> 3, oct = u & 7;
+    if constexpr (MODE == OZ_TRSM || MODE == OZ_INV2) {
+      const int ex = row >= T.nb ? 0 : 63 - (MODE == OZ_TRSM ? S.f[i0 + row] : S.tr[i0 + T.rb + row]);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[k] = to_fix(__longlong_as_double(w[k]), ex);
+    }
+    put_digits(pb, b_plane, row, oct, w);
+  };
+  const uint64_t da = smem_desc(smem_u32(pa)), db = smem_desc(smem_u32(pb));
+  // the products of sums s0 .. s1 (compile-time digit planes)
+  auto issue = [&](auto s0, auto s1) {
+#pragma unroll
+    for (int s = decltype(s0)::value; s <= decltype(s1)::value; ++s) {
+#pragma unroll
+      for (int i = 0; i <= s; ++i) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          mma_bf16(tmem + (uint32_t)((s & 3) * OT), da + (uint64_t)(i * (OPLANE >> 4) + 2 * k),
+                   db + (uint64_t)((s - i) * (b_plane >> 4) + 2 * k), idesc_f16(OT, BN),
+                   (i > 0 || k > 0) ? 1u : 0u);
       }
-      __syncwarp();
-    } else if (warp < drains) {
-      // ------------------------------------------- digit sums into 64 bits
-      for (int s = 0; s < SLICES && !dead; ++s) {
-        const int g = SLICES * ch + s, a = g & 3;
-        int ok = 1;
-        if (lane == 0) {
-          ok = oz_wait(&accF[a], (uint32_t)(g >> 2) & 1u, P.spin_cycles, abort_flag) ? 1 : 0;
+    }
+  };
+  long long acc[32];
+  bool dead = false;
+  constexpr bool one_chunk = MODE == OZ_TRSM || MODE == OZ_SYRK;
+  static_assert(OT * 8 == 2 * WT, "two units of a per thread, two (or one) of b");
+  for (int ch = 0; ch < (one_chunk ? 1 : T.kn); ++ch) {
+    const int kk = NB * (T.k0 + ch);
+    // -------------------------------------------------------- cut the operands
+    // the next unit's words are on their way while one is cut
+    {
+      long long w0[8], w1[8];
+      load_a(t, kk, w0);
+      load_a(t + WT, kk, w1);
+      put_a(t, w0);
+      load_b(t, kk, w0);
+      put_a(t + WT, w1);
+      if constexpr (BN == OT) load_b(t + WT, kk, w1);
+      put_b(t, w0);
+      if constexpr (BN == OT) put_b(t + WT, w1);
+    }
+    if (one_chunk || ch == 0) {
+#pragma unroll
+      for (int u = 0; u < 32; ++u) acc[u] = 0;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    // ---------------------------------------- products, digit sums into 64 bits
+    if (t == 0 && !dead) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      issue(Int<0>{}, Int<2>{});
+      mma_commit(&accF[0]);
+      issue(Int<3>{}, Int<3>{});
+    }
+    __syncwarp();
+    if (warp < drains) {
+      // sum s counts 2^(8 (6 - s)); modulo 2^64, so the first three only reach
+      // the upper word, and pairs of the others fit 32 bits
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        int ok = dead ? 0 : 1;
+        if (lane == 0 && !dead) {
+          ok = oz_wait(&accF[g], (uint32_t)ch & 1u, P.spin_cycles, abort_flag) ? 1 : 0;
           if (!ok && !*abort_flag) timed_out();
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) {
@@ -615,25 +756,61 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(const PrepArgs P, int arg)
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * OT + cg * 32);
-        const int sh = 8 * (SLICES - 1 - s);
+        const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * 32);
+        if (g == 0) {
 #pragma unroll
-        for (int hlf = 0; hlf < 2; ++hlf) {
-          uint32_t r[16];
-          tmem_ld16(ta + 16 * hlf, r);
-          tmem_wait_ld();
+          for (int c = 0; c < 32; c += 8) {
+            uint32_t r0[8], r1[8], r2[8];
+            tmem_ld8(ta + c, r0);
+            tmem_ld8(ta + OT + c, r1);
+            tmem_ld8(ta + 2 * OT + c, r2);
+            tmem_wait_ld();
 #pragma unroll
-          for (int u = 0; u < 16; ++u)
-            acc[16 * hlf + u] += (long long)__float2int_rn(__uint_as_float(r[u])) << sh;
+            for (int u = 0; u < 8; ++u) {
+              const uint32_t v = (((biased_int(r0[u]) << 8) + biased_int(r1[u])) << 8) + biased_int(r2[u]);
+              acc[c + u] += (long long)((unsigned long long)(
+                                v - ((OZ_BIAS << 16) + (OZ_BIAS << 8) + OZ_BIAS)) << 32);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < 32; c += 16) {
+            uint32_t r0[16], r1[16];
+            tmem_ld16(ta + (g == 1 ? 3 * OT : OT) + c, r0);
+            tmem_ld16(ta + (g == 1 ? 0 : 2 * OT) + c, r1);
+            tmem_wait_ld();
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const int lo = __float2int_rn(__uint_as_float(r1[u]));
+              if (g == 1)
+                acc[c + u] += (long long)((int)((biased_int(r0[u]) - OZ_BIAS) << 8) + lo) * 65536;
+              else
+                acc[c + u] += (long long)((int)(wide_int(r0[u]) << 8) + lo);
+            }
+          }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&accE[a]);
+        if (g == 0) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(accE);
+          if (t == 0) {   // accumulators 0 .. 2 again
+            if (oz_wait(accE, (uint32_t)ch & 1u, P.spin_cycles, abort_flag)) {
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              issue(Int<4>{}, Int<4>{});
+              mma_commit(&accF[1]);
+              issue(Int<5>{}, Int<6>{});
+              mma_commit(&accF[2]);
+            } else if (!*abort_flag) {
+              timed_out();
+            }
+          }
+          __syncwarp();
+        }
       }
     }
     __syncthreads();   // every MMA of the chunk is complete: its planes are free
   }
-  if (warp == WORKERS && lane == 0) {
+  if (t == 0) {
     mma_commit(done);
     if (!mbar_wait(done, 0, drain_limit)) timed_out();   // before anyone frees TMEM
   }
@@ -647,42 +824,57 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(const PrepArgs P, int arg)
       *reinterpret_cast<longlong2*>(o + u) = make_longlong2(acc[u], acc[u + 1]);
   }
   __syncthreads();
-  if (warp < WORKERS && !*abort_flag) {
-    for (int r = warp; r < T.na; r += WORKERS) {
-      const int er = MODE == OZ_INV1 ? S.xc[i0 + T.ra + r] : MODE == OZ_INV2 ? S.xr[i0 + arg + T.ra + r] : 0;
+  if (!*abort_flag) {
+    // a warp's eight rows, four at a time (old values in flight together)
 #pragma unroll
-      for (int cb = 0; cb < BN / 64; ++cb) {
-        const int c = 64 * cb + 2 * lane;
-        if (c >= T.nb) continue;
-        const longlong2 v = *reinterpret_cast<const longlong2*>(st + r * OUT_LD + c);
-        if constexpr (MODE == OZ_TRSM) {
-          const int f0 = min(max(S.f[i0 + c], 0), 62), f1 = min(max(S.f[i0 + c + 1], 0), 62);
-          *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + i0 + c) =
-              make_longlong2((long long)((unsigned long long)v.x << f0),
-                             (long long)((unsigned long long)v.y << f1));
-        } else if constexpr (MODE == OZ_SYRK) {
-          longlong2* p = reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + T.rb + c);
-          const longlong2 old = __ldcg(p);
-          *p = make_longlong2(old.x - v.x, old.y - v.y);
-        } else if constexpr (MODE == OZ_INV1) {
-          *reinterpret_cast<double2*>((double*)S.C + (int64_t)(i0 + T.ra + r) * ld + i0 + arg + T.rb + c) =
-              make_double2(from_fix(v.x, er - 62), from_fix(v.y, er - 62));
-        } else {
-          const int e0 = S.tr[i0 + T.rb + c], e1 = S.tr[i0 + T.rb + c + 1];
-          *reinterpret_cast<double2*>(S.X + (int64_t)(i0 + arg + T.ra + r) * ld + i0 + T.rb + c) =
-              make_double2(from_fix(-v.x, er + e0 - 62), from_fix(-v.y, er + e1 - 62));
-        }
+    for (int rr = 0; rr < OT / WORKERS; rr += 4) {
+      longlong2 old[4][BN / 64];
+      if constexpr (MODE == OZ_SYRK) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int cb = 0; cb < BN / 64; ++cb) {
+            const int r = warp + WORKERS * (rr + j), c = 64 * cb + 2 * lane;
+            if (r < T.na && c < T.nb)
+              old[j][cb] = __ldcg(reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + T.rb + c));
+          }
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int cb = 0; cb < BN / 64; ++cb) {
+          const int r = warp + WORKERS * (rr + j), c = 64 * cb + 2 * lane;
+          if (r >= T.na || c >= T.nb) continue;
+          const longlong2 v = *reinterpret_cast<const longlong2*>(st + r * OUT_LD + c);
+          if constexpr (MODE == OZ_TRSM) {
+            const int f0 = min(max(S.f[i0 + c] + 1, 0), 63), f1 = min(max(S.f[i0 + c + 1] + 1, 0), 63);
+            *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + i0 + c) =
+                make_longlong2((long long)((unsigned long long)v.x << f0),
+                               (long long)((unsigned long long)v.y << f1));
+          } else if constexpr (MODE == OZ_SYRK) {
+            *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + T.rb + c) =
+                make_longlong2(old[j][cb].x - 2 * v.x, old[j][cb].y - 2 * v.y);
+          } else if constexpr (MODE == OZ_INV1) {
+            const int er = S.xc[i0 + T.ra + r] - 62;
+            *reinterpret_cast<double2*>((double*)S.C + (int64_t)(i0 + T.ra + r) * ld + i0 + arg + T.rb + c) =
+                make_double2(from_fix(v.x, er), from_fix(v.y, er));
+          } else {
+            const int er = S.xr[i0 + arg + T.ra + r] - 62;
+            const int e0 = S.tr[i0 + T.rb + c], e1 = S.tr[i0 + T.rb + c + 1];
+            *reinterpret_cast<double2*>(S.X + (int64_t)(i0 + arg + T.ra + r) * ld + i0 + T.rb + c) =
+                make_double2(from_fix(-v.x, er + e0), from_fix(-v.y, er + e1));
+          }
+        }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == WORKERS)
+  if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
                  : "memory");
   if constexpr (MODE == OZ_SYRK) {
-    if (blockIdx.x == 0 && warp < WORKERS)
+    if (blockIdx.x == 0)
       potrf_block(S, arg + NB, *reinterpret_cast<PotrfSmem*>(smem), P.status);
   }
 }
@@ -849,7 +1041,7 @@ int prepare_impl(const float* A, const float* B, int m, int n, float damp, void*
   k_prep_scale<<<2, 1024, 0, s>>>(P);
   k_prep_load<<<dim3(dp / 32, dp / 32, 2), 256, 0, s>>>(P);
   BK_CUDA_OK(cudaGetLastError());
-  const dim3 oz(OZ_THREADS);
+  const dim3 oz(WT);
   BK_CUDA_OK(launch_pdl(k_prep_first, dim3(2), dim3(WT), sizeof(PotrfSmem), s, P));
   for (int k0 = 0; k0 + NB < dp; k0 += NB) {
     const unsigned nt = up(dp - k0 - NB, OT);
