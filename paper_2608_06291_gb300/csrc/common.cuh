@@ -80,16 +80,16 @@ struct FactorLayout {
 // (solve.cu); run after every write of the planes.
 int build_leaf_blocks(const FactorLayout& fl, char* factors, cudaStream_t s);
 
-// Solve workspace: [status 256 B][X mp x np][E^T hi, lo: np x mp each]
+// Solve workspace: [status 256 B][flags][X mp x np][E^T hi, lo: np x mp each]
 // [M hi, lo: mp x np each], fp32.  X holds W widened and, once an entry is
 // rounded, the value it was rounded at.  E^T is the error matrix transposed
 // (row = column index of W) so that it is K-major as the second operand of
 // M = L^B E; M is the stage-1 band product.  The M hi plane doubles as E^T in
 // fp32 for the leaves: a leaf block reads back only E tiles written inside the
 // block, and M is written only by band products, which run between blocks.
-// Then the leaves' dataflow words (one launch per block of leaves): a tile
-// counter per block, indexed by the block's first anti-diagonal, and a
-// readiness flag per padded tile; zeroed at the start of every solve.
+// The flags are the leaves' (one launch per block of leaves): a counter per block,
+// indexed by the block's first anti-diagonal, and a readiness flag per padded
+// tile; zeroed with the status at the start of every solve.
 constexpr int FLOW_COUNTERS = 8192;   // > the anti-diagonals of the largest problem (2 * 4096)
 struct SolveLayout {
   int64_t mp, np;
@@ -99,14 +99,14 @@ struct SolveLayout {
     np = round_up(n, PAD);
     const size_t plane = size_t(mp * np) * 4;
     off_status = 0;
-    off_X = 256;
+    off_flow = 256;
+    flow_bytes = size_t(FLOW_COUNTERS + (mp / TILE) * (np / TILE)) * 4;
+    off_X = align256(off_flow + flow_bytes);
     off_EtH = align256(off_X + plane);
     off_EtL = align256(off_EtH + plane);
     off_MH = align256(off_EtL + plane);
     off_ML = align256(off_MH + plane);
-    off_flow = align256(off_ML + plane);
-    flow_bytes = size_t(FLOW_COUNTERS + (mp / TILE) * (np / TILE)) * 4;
-    bytes = align256(off_flow + flow_bytes);
+    bytes = align256(off_ML + plane);
   }
 };
 

@@ -301,8 +301,8 @@ constexpr float LEAF_R = 12582912.f;
 __host__ __device__ constexpr int window_products(int P) { return 2 * P; }
 
 struct LeafSmem {
-  float Xs[TILE][TILE];                   // W after inbound updates
-  __align__(16) float LBs[TILE][36];      // stride 36: conflict-free float4 row reads
+  float Xs[TILE + 1][TILE];               // W after inbound updates (row TILE: zeros)
+  __align__(16) float LBs[TILE + 1][36];  // stride 36: conflict-free float4 row reads (row TILE: zeros)
   __align__(16) float LA0[TILE][KM];      // LA0[j][q] = L^A[J,J][q][j]
   float T1s[TILE][TILE + 1];              // T1, the initial G of a window-P leaf (P >= 1)
   __align__(16) float Ebr[4][LEAF_ROWS_PADDED];   // errors of a step, by row (ring of 4 steps)
@@ -319,10 +319,10 @@ struct LeafSmem {
     } pro;
     struct {   // the wavefront
       float EsT[TILE][TILE + 1];              // after the wavefront: E transposed
-      __align__(8) float2 XE[TILE][TILE];     // (pre-rounding value, error)
-      uint8_t Cs[TILE][TILE];
+      float Xd[2 * TILE][TILE];               // pre-rounding value of step d, column q
     } w;
   } u;
+  __device__ __forceinline__ float& xd(int d, int q) { return u.w.Xd[d][q]; }
 };
 
 // C[r][c] = sum_k At[k][r] B(k, c) for the 4 x 2 block of thread t < 128
@@ -426,6 +426,198 @@ __device__ __forceinline__ void flow_wait(const FlowCtx& fc, int I1, int J1, int
   leaf_sync();
 }
 
+// ---------------------------------------------------------- the wavefront
+// Steps go in intervals of two (steps 2k and 2k+1) with one barrier at the
+// end of each.  In interval k the helpers fold the errors of steps 2k-2 and
+// 2k-1 (published at the barrier before it) and leave the partial pre of
+// steps 2k+2 and 2k+3, so the pre of step d covers the errors of steps up
+// to d-3 (d even) or d-4 (d odd).  The chain adds the rest itself: every
+// error of the last two (three) steps that reaches (p, q), i.e. entry
+// (p-a, q-b) for 1 <= a+b <= 2 (3), with weight L^B[p][p-a] L^A[q][q-b].
+// Its own column's errors it keeps in registers (E1..E3: steps d-1..d-3);
+// those of the columns to its left (L1_*: column q-1, L2_*: q-2, L3_3:
+// q-3, each from the step its suffix names back) arrive by shuffles, and
+// only L1_1, the left neighbour's newest error, is on the critical path.
+// What the wavefront of a tile reads and leaves in shared memory are fields of the
+// same names in LeafSmem and StripSmem; warps 0 .. 3 of a CTA, synchronised by
+// leaf_sync.
+
+// The chain (warp 0) over the tile at (r0, c0) of an m x n problem.
+template <class SM>
+__device__ __forceinline__ void wave_chain(SM& S, const float (*LA0)[KM], int64_t r0, int64_t c0, int m, int n,
+                                       long long* clk) {
+  const int lane = threadIdx.x & 31, q = lane;
+  // ------------------------------------------------ the chain
+  const bool col_real = (c0 + q) < n;
+  const int rows_real = m - (int)r0;     // rows p < rows_real are inside W
+  // entry (p, q) is real iff 0 <= p < plim (one unsigned compare per step)
+  const unsigned plim = col_real ? (unsigned)min(max(rows_real, 0), TILE) : 0u;
+  const float la1 = q >= 1 ? LA0[q - 1][q] : 0.f;
+  const float la2 = q >= 2 ? LA0[q - 2][q] : 0.f;
+  const float la3 = q >= 3 ? LA0[q - 3][q] : 0.f;
+  constexpr float R = LEAF_R;
+  float E1 = 0.f, E2 = 0.f, E3 = 0.f;
+  float L1_1 = 0.f, L1_2 = 0.f, L1_3 = 0.f, L2_2 = 0.f, L2_3 = 0.f, L3_3 = 0.f;
+  // One step.  Of the explicit terms only E1 (own column, last step) and
+  // L1_1 (left neighbour, last step, still in flight from its shuffle) are
+  // new; the sum of the older ones is formed first so that these two enter
+  // last.  The shuffles the next step needs are issued as soon as their
+  // inputs exist.  Entries off the tile or outside W get a zero error (the
+  // factor mk).
+  auto step = [&](int d, bool odd, float pre, const float4& g, const float4& lb) {
+    const int p = d - q;
+    float A = fmaf(la2, L2_2, pre);
+    const float A2 = fmaf(lb.y, E2, (lb.x * la1) * L1_2);
+    if (odd) {
+      const float o1 = fmaf(la3, L3_3, (lb.x * la2) * L2_3);
+      const float o2 = fmaf(lb.y * la1, L1_3, lb.z * E3);
+      A = A + (o1 + o2);
+    }
+    A = A + A2;
+    float nL3_3 = 0.f;   // column q-3, this step's d-2: an odd step reads it
+    if (!odd) nL3_3 = __shfl_up_sync(0xffffffffu, L2_2, 1);
+    const float x = fmaf(la1, L1_1, fmaf(lb.x, E1, A));
+    const float nL2_2 = __shfl_up_sync(0xffffffffu, L1_1, 1);   // column q-2, step d-1
+    const float tc = fminf(fmaxf(fmaf(x, g.y, R), g.z), g.w);
+    const float e = (unsigned)p < plim ? fmaf(g.x, tc - R, -x) : 0.f;   // s (c - z) - x, rounded once
+    L1_3 = L1_2;
+    L1_2 = L1_1;
+    L2_3 = L2_2;
+    L2_2 = nL2_2;
+    L3_3 = nL3_3;
+    E3 = E2;
+    E2 = E1;
+    E1 = e;
+    L1_1 = __shfl_up_sync(0xffffffffu, e, 1);                    // column q-1, step d
+    S.xd(d, q) = x;
+    S.Ebr[d & 3][p & (TILE - 1)] = e;    // rows off the tile get a zero
+  };
+  // the grid and the sub-diagonal L^B of the next interval's entries are
+  // loaded one interval ahead; two intervals per loop iteration (in k_strips
+  // 173 cycles a step, against 188 with one and 194 with three or six: the three
+  // teams' loops share the instruction caches)
+  float4 g0 = S.Srzl[(0 - q) & (TILE - 1)][q], g1 = S.Srzl[(1 - q) & (TILE - 1)][q];
+  float4 lb0 = S.Lsub[(0 - q) & (TILE - 1)], lb1 = S.Lsub[(1 - q) & (TILE - 1)];
+  leaf_sync();   // the helpers' pre of steps 0 and 1
+  if (clk != nullptr && lane == 0) clk[0] = clock64();
+#pragma unroll 2
+  for (int k = 0; k < TILE; ++k) {
+    const int d0 = 2 * k, d1 = 2 * k + 1;
+    const float* pa = &S.Part[d0 & 3][0][q];
+    const float* pb = &S.Part[d1 & 3][0][q];
+    static_assert(LEAF_HELPERS == 3, "the chain sums three partials");
+    const float pre0 = (pa[0] + pa[TILE]) + pa[2 * TILE];
+    const float pre1 = (pb[0] + pb[TILE]) + pb[2 * TILE];
+    const float4 g0c = g0, g1c = g1, lb0c = lb0, lb1c = lb1;
+    const int n0 = (d0 + 2 - q) & (TILE - 1), n1 = (d1 + 2 - q) & (TILE - 1);
+    g0 = S.Srzl[n0][q];
+    g1 = S.Srzl[n1][q];
+    lb0 = S.Lsub[n0];
+    lb1 = S.Lsub[n1];
+    step(d0, false, pre0, g0c, lb0c);
+    if (d1 < 2 * TILE - 1) step(d1, true, pre1, g1c, lb1c);
+    leaf_sync();
+  }
+  if (clk != nullptr && lane == 0) clk[1] = clock64();
+}
+
+// Helper g (warp g + 1): rows 12 g .. 12 g + 11 of G for column q = lane, from T1
+// (HAS_T1) or zero; final_g: complete on return.
+template <bool HAS_T1, class SM>
+__device__ __forceinline__ void wave_helper(SM& S, const float (*LA0)[KM], int g, int q, bool final_g,
+                                        float (&Gg)[LEAF_ROWS_PER_HELPER]) {
+  // ------------------------------------------------ helpers: rows i0..i0+11
+  const int i0 = LEAF_ROWS_PER_HELPER * g;
+  // L^A[q][j] sits in slot (j + 2 + i0 - 8b) mod 32 during steps [8b, 8b + 8)
+  // (intervals 4b .. 4b+3): the column j = s - i0 - r of row i0 + r that
+  // step s = 8b + 2v - 2 (+1) brings is in slot 2v - r (+1) mod 32
+  float LAr[TILE];
+#pragma unroll
+  for (int sl = 0; sl < TILE; ++sl) LAr[sl] = LA0[(sl - 2 - i0) & (TILE - 1)][q];
+#pragma unroll
+  for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
+    Gg[r] = (HAS_T1 && i0 + r < TILE) ? S.T1s[i0 + r][q] : 0.f;
+  // The L^B row (and, for helper 0, X) of step d's entry (row d - q), zero
+  // off the tile; loaded one interval before use into one of four slots
+  // (slots 2, 3 serve even intervals, 0, 1 odd ones).
+  float LBv[4][LEAF_ROWS_PER_HELPER], Xv[4];
+  auto fetch = [&](int d, int slot) {
+    const int pr = (int)min((unsigned)(d - q), (unsigned)TILE);   // off the tile: the zero row
+#pragma unroll
+    for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v) {
+      const float4 l = *reinterpret_cast<const float4*>(&S.LBs[pr][i0 + 4 * v]);
+      LBv[slot][4 * v] = l.x;
+      LBv[slot][4 * v + 1] = l.y;
+      LBv[slot][4 * v + 2] = l.z;
+      LBv[slot][4 * v + 3] = l.w;
+    }
+    Xv[slot] = g == 0 ? S.Xs[pr][q] : 0.f;
+  };
+  // partial pre of step d's entry over these rows (zero off the tile)
+  auto dot = [&](int d, int slot) {
+    float a4[LEAF_ROWS_PER_HELPER / 4];
+#pragma unroll
+    for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v)
+      a4[v] = fmaf(LBv[slot][4 * v], Gg[4 * v],
+                   fmaf(LBv[slot][4 * v + 1], Gg[4 * v + 1],
+                        fmaf(LBv[slot][4 * v + 2], Gg[4 * v + 2],
+                             fmaf(LBv[slot][4 * v + 3], Gg[4 * v + 3], v == 0 ? Xv[slot] : 0.f))));
+    static_assert(LEAF_ROWS_PER_HELPER == 12, "three float4 groups per helper");
+    S.Part[d & 3][g][q] = (a4[0] + a4[1]) + a4[2];
+  };
+  // fold the errors of step sidx (its row i0 + r came from column sidx - i0 - r)
+  auto fold = [&](int sidx, int slot0) {
+    float ev[LEAF_ROWS_PER_HELPER];
+#pragma unroll
+    for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v) {
+      const float4 e4 = *reinterpret_cast<const float4*>(&S.Ebr[sidx & 3][i0 + 4 * v]);
+      ev[4 * v] = e4.x;
+      ev[4 * v + 1] = e4.y;
+      ev[4 * v + 2] = e4.z;
+      ev[4 * v + 3] = e4.w;
+    }
+#pragma unroll
+    for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
+      Gg[r] = fmaf(ev[r], LAr[(slot0 - r) & (TILE - 1)], Gg[r]);
+  };
+  // the pre of steps 0 and 1: nothing folded yet
+  fetch(0, 0);
+  fetch(1, 1);
+  dot(0, 0);
+  dot(1, 1);
+  fetch(2, 2);
+  fetch(3, 3);
+  leaf_sync();   // the chain's interval 0 may start
+#pragma unroll 1
+  for (int b = 0; b < TILE / 4; ++b) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int k = 4 * b + v;
+      const int cur = (v & 1) ? 0 : 2, nxt = (v & 1) ? 2 : 0;
+      fetch(2 * k + 4, nxt);    // rows of the next interval, ahead of their use
+      fetch(2 * k + 5, nxt + 1);
+      if (k >= 1) {             // steps 2k-2 and 2k-1 were published at the last barrier
+        fold(2 * k - 2, 2 * v);
+        fold(2 * k - 1, 2 * v + 1);
+      }
+      if (2 * k + 2 < 2 * TILE - 1) dot(2 * k + 2, cur);
+      if (2 * k + 3 < 2 * TILE - 1) dot(2 * k + 3, cur + 1);
+      leaf_sync();
+    }
+    // next block: the slot of every column drops by 8, i.e. new slot s = old slot s + 8
+    float tmp[TILE];
+#pragma unroll
+    for (int j = 0; j < TILE; ++j) tmp[j] = LAr[(j + 8) & (TILE - 1)];
+#pragma unroll
+    for (int j = 0; j < TILE; ++j) LAr[j] = tmp[j];
+  }
+  if (final_g) {
+    // the last step's errors too (published at the last barrier; LAr is back at
+    // its first rotation): G[i][q] = T1[i][q] + sum_{j <= q} E[i][j] L^A[J,J][q][j]
+    fold(2 * TILE - 2, 0);
+  }
+}
+
 // Rounds tile (I, J); run by threads 0 .. LEAF_THREADS-1 of the CTA.  With
 // PDL, the factor blocks and the grid (read-only during the solve, the grid
 // written by the solve's first kernel, more than one kernel ago), and the
@@ -464,6 +656,8 @@ __device__ __forceinline__ void leaf_tile(const LeafArgs& a, int I, int J, LeafS
   const float* lak = a.LAblk + (int64_t)J * LEAF_BLOCKS * LEAF_BLOCK_FLOATS;
   copy_block(&S.LBs[0][0], lbk, t);
   copy_block(&S.LA0[0][0], lak, t);
+  if (t < 36) S.LBs[TILE][t] = 0.f;
+  if (t < TILE) S.Xs[TILE][t] = 0.f;
   // The window.  N_d of this tile (the errors of row I - d of the window
   // seen from column block J) equals the final G of tile (I - d, J), which
   // sits at position P - d of the same block: every leaf leaves its final G
@@ -615,200 +809,30 @@ __device__ __forceinline__ void leaf_tile(const LeafArgs& a, int I, int J, LeafS
     S.Lsub[t] = make_float4(t >= 1 ? S.LBs[t][t - 1] : 0.f, t >= 2 ? S.LBs[t][t - 2] : 0.f,
                             t >= 3 ? S.LBs[t][t - 3] : 0.f, 0.f);
   leaf_sync();
-  // ---------------------------------------------------------- the wavefront
-  // Steps go in intervals of two (steps 2k and 2k+1) with one barrier at the
-  // end of each.  In interval k the helpers fold the errors of steps 2k-2 and
-  // 2k-1 (published at the barrier before it) and leave the partial pre of
-  // steps 2k+2 and 2k+3, so the pre of step d covers the errors of steps up
-  // to d-3 (d even) or d-4 (d odd).  The chain adds the rest itself: every
-  // error of the last two (three) steps that reaches (p, q), i.e. entry
-  // (p-a, q-b) for 1 <= a+b <= 2 (3), with weight L^B[p][p-a] L^A[q][q-b].
-  // Its own column's errors it keeps in registers (E1..E3: steps d-1..d-3);
-  // those of the columns to its left (L1_*: column q-1, L2_*: q-2, L3_3:
-  // q-3, each from the step its suffix names back) arrive by shuffles, and
-  // only L1_1, the left neighbour's newest error, is on the critical path.
-  const int q = lane;
+  // the wavefront (wave_chain, wave_helper)
   if (w == 0) {
-    // ------------------------------------------------ the chain
-    const bool col_real = (c0 + q) < a.n;
-    const int rows_real = a.m - (int)r0;     // rows p < rows_real are inside W
-    // entry (p, q) is real iff 0 <= p < plim (one unsigned compare per step)
-    const unsigned plim = col_real ? (unsigned)min(max(rows_real, 0), TILE) : 0u;
-    const float la1 = q >= 1 ? S.LA0[q - 1][q] : 0.f;
-    const float la2 = q >= 2 ? S.LA0[q - 2][q] : 0.f;
-    const float la3 = q >= 3 ? S.LA0[q - 3][q] : 0.f;
-    constexpr float R = LEAF_R;
-    float E1 = 0.f, E2 = 0.f, E3 = 0.f;
-    float L1_1 = 0.f, L1_2 = 0.f, L1_3 = 0.f, L2_2 = 0.f, L2_3 = 0.f, L3_3 = 0.f;
-    // One step.  Of the explicit terms only E1 (own column, last step) and
-    // L1_1 (left neighbour, last step, still in flight from its shuffle) are
-    // new; the sum of the older ones is formed first so that these two enter
-    // last.  The shuffles the next step needs are issued as soon as their
-    // inputs exist.  Entries off the tile or outside W get a zero error (the
-    // factor mk).
-    auto step = [&](int d, bool odd, float pre, const float4& g, const float4& lb) {
-      const int p = d - q;
-      const bool on_tile = (unsigned)p < (unsigned)TILE;
-      float A = fmaf(la2, L2_2, pre);
-      const float A2 = fmaf(lb.y, E2, (lb.x * la1) * L1_2);
-      if (odd) {
-        const float o1 = fmaf(la3, L3_3, (lb.x * la2) * L2_3);
-        const float o2 = fmaf(lb.y * la1, L1_3, lb.z * E3);
-        A = A + (o1 + o2);
-      }
-      A = A + A2;
-      const float nL3_3 = __shfl_up_sync(0xffffffffu, L2_2, 1);   // column q-3, this step's d-2
-      const float x = fmaf(la1, L1_1, fmaf(lb.x, E1, A));
-      const float nL2_2 = __shfl_up_sync(0xffffffffu, L1_1, 1);   // column q-2, step d-1
-      const float tc = fminf(fmaxf(fmaf(x, g.y, R), g.z), g.w);
-      const float mk = (unsigned)p < plim ? 1.f : 0.f;
-      const float e = fmaf(g.x, tc - R, -x) * mk;   // s (c - z) - x, rounded once
-      L1_3 = L1_2;
-      L1_2 = L1_1;
-      L2_3 = L2_2;
-      L2_2 = nL2_2;
-      L3_3 = nL3_3;
-      E3 = E2;
-      E2 = E1;
-      E1 = e;
-      L1_1 = __shfl_up_sync(0xffffffffu, e, 1);                    // column q-1, step d
-      if (on_tile) {
-        S.u.w.XE[p][q] = make_float2(x, e);
-        S.u.w.Cs[p][q] = (uint8_t)(int)(tc - g.z);
-      }
-      S.Ebr[d & 3][p & (TILE - 1)] = e;    // rows off the tile get a zero
-    };
-    // the grid and the sub-diagonal L^B of the next interval's entries are
-    // loaded one interval ahead; three intervals per loop iteration, so that
-    // the three-step histories (E*, L*_*) rotate by renaming
-    float4 g0 = S.Srzl[(0 - q) & (TILE - 1)][q], g1 = S.Srzl[(1 - q) & (TILE - 1)][q];
-    float4 lb0 = S.Lsub[(0 - q) & (TILE - 1)], lb1 = S.Lsub[(1 - q) & (TILE - 1)];
-    leaf_sync();   // the helpers' pre of steps 0 and 1
-    if (a.clk != nullptr && lane == 0) a.clk[0] = clock64();
-#pragma unroll 3
-    for (int k = 0; k < TILE; ++k) {
-      const int d0 = 2 * k, d1 = 2 * k + 1;
-      const float* pa = &S.Part[d0 & 3][0][q];
-      const float* pb = &S.Part[d1 & 3][0][q];
-      static_assert(LEAF_HELPERS == 3, "the chain sums three partials");
-      const float pre0 = (pa[0] + pa[TILE]) + pa[2 * TILE];
-      const float pre1 = (pb[0] + pb[TILE]) + pb[2 * TILE];
-      const float4 g0c = g0, g1c = g1, lb0c = lb0, lb1c = lb1;
-      const int n0 = (d0 + 2 - q) & (TILE - 1), n1 = (d1 + 2 - q) & (TILE - 1);
-      g0 = S.Srzl[n0][q];
-      g1 = S.Srzl[n1][q];
-      lb0 = S.Lsub[n0];
-      lb1 = S.Lsub[n1];
-      step(d0, false, pre0, g0c, lb0c);
-      if (d1 < 2 * TILE - 1) step(d1, true, pre1, g1c, lb1c);
-      leaf_sync();
-    }
-    if (a.clk != nullptr && lane == 0) a.clk[1] = clock64();
+    wave_chain(S, S.LA0, r0, c0, a.m, a.n, a.clk);
   } else {
-    // ------------------------------------------------ helpers: rows i0..i0+11
-    const int g = w - 1, i0 = LEAF_ROWS_PER_HELPER * g;
-    // L^A[q][j] sits in slot (j + 2 + i0 - 8b) mod 32 during steps [8b, 8b + 8)
-    // (intervals 4b .. 4b+3): the column j = s - i0 - r of row i0 + r that
-    // step s = 8b + 2v - 2 (+1) brings is in slot 2v - r (+1) mod 32
-    float LAr[TILE];
-#pragma unroll
-    for (int sl = 0; sl < TILE; ++sl) LAr[sl] = S.LA0[(sl - 2 - i0) & (TILE - 1)][q];
     float Gg[LEAF_ROWS_PER_HELPER];
-#pragma unroll
-    for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
-      Gg[r] = (P >= 1 && i0 + r < TILE) ? S.T1s[i0 + r][q] : 0.f;
-    // The L^B row (and, for helper 0, X) of step d's entry (row d - q), zero
-    // off the tile; loaded one interval before use into one of four slots
-    // (slots 2, 3 serve even intervals, 0, 1 odd ones).
-    float LBv[4][LEAF_ROWS_PER_HELPER], Xv[4];
-    auto fetch = [&](int d, int slot) {
-      const int pn = d - q;
-      const bool on_tile = pn >= 0 && pn < TILE;
-      const int pr = on_tile ? pn : 0;
-#pragma unroll
-      for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v) {
-        float4 l = *reinterpret_cast<const float4*>(&S.LBs[pr][i0 + 4 * v]);
-        if (!on_tile) l = make_float4(0.f, 0.f, 0.f, 0.f);
-        LBv[slot][4 * v] = l.x;
-        LBv[slot][4 * v + 1] = l.y;
-        LBv[slot][4 * v + 2] = l.z;
-        LBv[slot][4 * v + 3] = l.w;
-      }
-      Xv[slot] = (g == 0 && on_tile) ? S.Xs[pr][q] : 0.f;
-    };
-    // partial pre of step d's entry over these rows (zero off the tile)
-    auto dot = [&](int d, int slot) {
-      float a4[LEAF_ROWS_PER_HELPER / 4];
-#pragma unroll
-      for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v)
-        a4[v] = fmaf(LBv[slot][4 * v], Gg[4 * v],
-                     fmaf(LBv[slot][4 * v + 1], Gg[4 * v + 1],
-                          fmaf(LBv[slot][4 * v + 2], Gg[4 * v + 2],
-                               fmaf(LBv[slot][4 * v + 3], Gg[4 * v + 3], v == 0 ? Xv[slot] : 0.f))));
-      static_assert(LEAF_ROWS_PER_HELPER == 12, "three float4 groups per helper");
-      S.Part[d & 3][g][q] = (a4[0] + a4[1]) + a4[2];
-    };
-    // fold the errors of step sidx (its row i0 + r came from column sidx - i0 - r)
-    auto fold = [&](int sidx, int slot0) {
-      float ev[LEAF_ROWS_PER_HELPER];
-#pragma unroll
-      for (int v = 0; v < LEAF_ROWS_PER_HELPER / 4; ++v) {
-        const float4 e4 = *reinterpret_cast<const float4*>(&S.Ebr[sidx & 3][i0 + 4 * v]);
-        ev[4 * v] = e4.x;
-        ev[4 * v + 1] = e4.y;
-        ev[4 * v + 2] = e4.z;
-        ev[4 * v + 3] = e4.w;
-      }
-#pragma unroll
-      for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
-        Gg[r] = fmaf(ev[r], LAr[(slot0 - r) & (TILE - 1)], Gg[r]);
-    };
-    // the pre of steps 0 and 1: nothing folded yet
-    fetch(0, 0);
-    fetch(1, 1);
-    dot(0, 0);
-    dot(1, 1);
-    fetch(2, 2);
-    fetch(3, 3);
-    leaf_sync();   // the chain's interval 0 may start
-#pragma unroll 1
-    for (int b = 0; b < TILE / 4; ++b) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const int k = 4 * b + v;
-        const int cur = (v & 1) ? 0 : 2, nxt = (v & 1) ? 2 : 0;
-        fetch(2 * k + 4, nxt);    // rows of the next interval, ahead of their use
-        fetch(2 * k + 5, nxt + 1);
-        if (k >= 1) {             // steps 2k-2 and 2k-1 were published at the last barrier
-          fold(2 * k - 2, 2 * v);
-          fold(2 * k - 1, 2 * v + 1);
-        }
-        if (2 * k + 2 < 2 * TILE - 1) dot(2 * k + 2, cur);
-        if (2 * k + 3 < 2 * TILE - 1) dot(2 * k + 3, cur + 1);
-        leaf_sync();
-      }
-      // next block: the slot of every column drops by 8, i.e. new slot s = old slot s + 8
-      float tmp[TILE];
-#pragma unroll
-      for (int j = 0; j < TILE; ++j) tmp[j] = LAr[(j + 8) & (TILE - 1)];
-#pragma unroll
-      for (int j = 0; j < TILE; ++j) LAr[j] = tmp[j];
-    }
+    wave_helper<(P >= 1)>(S, S.LA0, w - 1, lane, P < LEAF_WINDOW, Gg);
     if (P < LEAF_WINDOW) {
-      // the final G (the last step's errors, published at the last barrier,
-      // folded too; LAr is back at its first rotation) for the tiles below
-      // in this block: G[i][q] = T1[i][q] + sum_{j <= q} E[i][j] L^A[J,J][q][j]
-      fold(2 * TILE - 2, 0);
+      const int i0 = LEAF_ROWS_PER_HELPER * (w - 1);
 #pragma unroll
       for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
-        if (i0 + r < TILE) a.Gout[(r0 + i0 + r) * a.ldx + c0 + q] = Gg[r];
+        if (i0 + r < TILE) a.Gout[(r0 + i0 + r) * a.ldx + c0 + lane] = Gg[r];
     }
   }
   leaf_sync();   // the wavefront is done: its arrays are free
   // transpose E through a padded buffer (conflict-free both ways)
   for (int e = t; e < TILE * TILE; e += LEAF_THREADS) {
     const int r = e / TILE, c = e % TILE;
-    S.u.w.EsT[c][r] = S.u.w.XE[r][c].y;
+    // the chain's rounding again, from its pre-rounding value: code and error
+    const float x = S.u.w.Xd[r + c][c];
+    const float4 g = S.Srzl[r][c];
+    const float tc = fminf(fmaxf(fmaf(x, g.y, LEAF_R), g.z), g.w);
+    const bool real = (r0 + r) < a.m && (c0 + c) < a.n;
+    S.u.w.EsT[c][r] = real ? fmaf(g.x, tc - LEAF_R, -x) : 0.f;
+    if (real) a.codes[(r0 + r) * a.n + c0 + c] = (uint8_t)(int)(tc - g.z);
   }
   leaf_sync();
   if constexpr (MODE == LEAF_FLOW) {
@@ -827,10 +851,9 @@ __device__ __forceinline__ void leaf_tile(const LeafArgs& a, int I, int J, LeafS
   bool bad = false;
   for (int e = t; e < TILE * TILE; e += LEAF_THREADS) {
     const int r = e / TILE, c = e % TILE;
-    const float xr = S.u.w.XE[r][c].x;
+    const float xr = S.u.w.Xd[r + c][c];
     bad |= !isfinite(xr);
     a.X[(r0 + r) * a.ldx + c0 + c] = xr;
-    if ((r0 + r) < a.m && (c0 + c) < a.n) a.codes[(r0 + r) * a.n + c0 + c] = S.u.w.Cs[r][c];
     const float ev = S.u.w.EsT[r][c];        // E^T row c0 + r, column r0 + c
     const float hi = tf32_hi(ev);
     const int64_t o = (c0 + r) * a.ldt + r0 + c;
@@ -897,6 +920,485 @@ __global__ void __launch_bounds__(LEAF_THREADS) k_leaf_heads(int K, const __grid
   a.zeros = L.zeros[h];
   const int I = max(0, K - (a.Nt - 1)) + blockIdx.x;
   leaf_tile<LEAF_PDL, P>(a, I, K - I, S);
+}
+
+// ------------------------------------------------------- blocks of leaves
+// All leaves of anti-diagonals [k, k + nb) (nb <= LEAF_WINDOW + 1) in one
+// launch, one CTA per 32-row strip: strip I rounds its tiles (I, k + t - I), t = 0
+// .. nb - 1, one after the other.  Tile t needs its left neighbour's errors, which
+// are the CTA's own, and the final G of the tile above it, (I - 1, J), which strip
+// I - 1 rounded at t - 1: adjacent strips are the CTAs of a cluster, and a strip
+// writes its final G straight into the shared memory of the strip below
+// (double-buffered, an mbarrier each way).  Between clusters, and for the rows
+// further up that a window reads, G goes through global memory and a flag per
+// tile; a strip that waits for a flag delays only what is below it, one tile later
+// per strip, so a block pays that latency about once.
+//
+// Three teams of four warps: the wavefront team (chain and helpers) rounds tile t;
+// meanwhile the errors' team writes tile t - 1 out and sums T1's terms of tile t + 1
+// (see leaf_tile) from the strip's own errors, and the upper team sums U's from the
+// G of the strips above and loads the grid and X; both up to the terms of the two
+// neighbours, which they add between the tiles.
+//
+// One launch per anti-diagonal cost 9.6 us each at 4096 x 4096, of which the
+// 63 steps alone take 5.4: the rest was the launch boundary, the neighbours' tiles
+// from L2, set-up and the way out, and the next launch's window products beside the
+// wavefront.  Here about 7.8 (4096^2 solve 4.68 -> 4.22 ms, 4096 x 11008 12.48 ->
+// 11.29): 2 000 cycles between two tiles (G's copy 400, a product 900, the errors
+// 900), and a wavefront of 13 to 17 thousand, which the other teams' products still
+// stretch.
+constexpr int STRIP_TEAM = LEAF_THREADS;             // threads of a team
+constexpr int STRIP_THREADS = 3 * STRIP_TEAM;       // 12 warps: 168 registers a thread
+constexpr int STRIP_CLUSTER = 8;                     // strips of a cluster, at most
+
+struct StripSmem {
+  __align__(16) float4 Srzl[TILE][TILE];
+  __align__(16) float LBs[TILE + 1][36];
+  float4 Lsub[TILE];
+  __align__(16) float LB1[TILE][KM];                 // L^B[I, I-1], k-major
+  __align__(16) float LA0[2][TILE][KM];              // L^A[J, J] of tiles t, t + 1
+  __align__(16) float LA1[TILE][KM];                 // L^A[J, J-1] of the next tile
+  __align__(16) float Gin[2][TILE][KM];              // final G of the tile above, by tile parity
+  __align__(16) float Gs[2][LEAF_ROWS_PADDED][KM];   // our own on its way down
+  __align__(16) float Es[TILE][KM];                  // errors of the last tile, k-major: [j][i]
+  float Xs[TILE + 1][TILE];
+  float T1s[TILE][TILE + 1];
+  float Xd[2 * TILE][TILE];
+  __align__(16) float Ebr[4][LEAF_ROWS_PADDED];
+  float Part[4][LEAF_HELPERS][TILE];
+  // the window's operands, one d at a time, double-buffered (see LeafSmem)
+  __align__(16) float B[2][4][TILE][KM];
+  unsigned long long gfull[2], gfree[2];             // mbarriers of Gin (ours), of the strip below's
+  int claim;
+  __device__ __forceinline__ float& xd(int d, int q) { return Xd[d][q]; }
+};
+
+struct StripArgs {
+  int k, nb;
+  int ilo, nstrips;      // strips ilo .. ilo + nstrips - 1
+  int cs;                // CTAs of a cluster
+  FlowCtx fc;
+  unsigned* claim;       // clusters started (zero before the launch)
+};
+
+__device__ __forceinline__ uint32_t sh_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ uint32_t peer_u32(const void* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(sh_u32(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void strip_sync() { asm volatile("bar.sync 0;" ::: "memory"); }
+template <int BAR>   // 3: the errors' team, 4: the upper team
+__device__ __forceinline__ void team_sync() {
+  asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(STRIP_TEAM) : "memory");
+}
+
+// Bounded wait for the phase of an mbarrier by one thread, and by lane 0 of a warp
+// that meets after it.  Past `limit` the time-out is
+// recorded, but the phase is waited for on (about 2 s at most): the other side
+// always gets there, and a phase that is still open may neither be armed again nor
+// have its copies left in flight.  False if even that ran out.
+__device__ __forceinline__ bool strip_wait1(unsigned long long* bar, uint32_t parity, long long limit,
+                                            int* status) {
+  const long long t0 = clock64();
+  bool late = false;
+  while (true) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(sh_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    const long long dt = clock64() - t0;
+    if (dt > limit && !late) {
+      late = true;
+      raise_status(status, BAKRON_ERR_TIMEOUT);
+    }
+    if (dt > limit && dt > 4000000000LL) return false;
+  }
+}
+__device__ __forceinline__ bool strip_wait(unsigned long long* bar, uint32_t parity, long long limit,
+                                           int* status) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0) ok = strip_wait1(bar, parity, limit, status) ? 1 : 0;
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;   // the same for the whole warp
+}
+__device__ __forceinline__ void strip_arrive(unsigned long long* bar, int rank) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_u32(bar, rank))
+               : "memory");
+}
+// Bounded wait for a tile's flag, by one thread.
+__device__ __forceinline__ void flag_wait(const FlowCtx& fc, int I, int J, int* status) {
+  const unsigned* f = fc.done + (int64_t)I * fc.ntp + J;
+  const long long t0 = clock64();
+  while (!ld_acquire_u32(f)) {
+    if (clock64() - t0 > fc.spin_cycles) {
+      raise_status(status, BAKRON_ERR_TIMEOUT);
+      break;
+    }
+    __nanosleep(32);
+  }
+}
+
+// T += At^T B of one 32^3 product, thread t's rows pr .. pr + 3, columns pc, pc + 1
+// (k ascending): At[k][row], B[k][column], both with row stride KM.
+__device__ __forceinline__ void strip_product(const float (*At)[KM], const float (*B)[KM], int pr, int pc,
+                                              float (&acc)[4][2]) {
+#pragma unroll 8
+  for (int k = 0; k < TILE; ++k) {
+    const float4 a = *reinterpret_cast<const float4*>(&At[k][pr]);
+    const float2 b = *reinterpret_cast<const float2*>(&B[k][pc]);
+    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[i][0] = fmaf(av[i], b.x, acc[i][0]);
+      acc[i][1] = fmaf(av[i], b.y, acc[i][1]);
+    }
+  }
+}
+
+__device__ __forceinline__ void strip_body(const LeafArgs& a, const StripArgs& s) {
+  extern __shared__ __align__(16) unsigned char leaf_smem[];
+  StripSmem& S = *reinterpret_cast<StripSmem*>(leaf_smem);
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int rank = (int)blockIdx.x % s.cs;           // clusters lie along x
+  if (t == 0) {
+    for (int b = 0; b < 2; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sh_u32(&S.gfull[b])), "r"(1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sh_u32(&S.gfree[b])), "r"(1));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (rank == 0) {
+      // clusters take their strips in the order they start, so the strips above
+      // are held by clusters that run or have run
+      const unsigned c = atomicAdd(s.claim, 1u);
+      for (int r = 0; r < s.cs; ++r)
+        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(peer_u32(&S.claim, r)), "r"(c)
+                     : "memory");
+    }
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  const int I = s.ilo + S.claim * s.cs + rank, iend = s.ilo + s.nstrips;
+  const int64_t r0 = (int64_t)I * TILE;
+  const int tb = max(0, I - s.k), te = I < iend ? min(s.nb, a.Nt + I - s.k) : tb;   // tiles t in [tb, te)
+  const bool live = te > tb;
+  const int vt = t & (STRIP_TEAM - 1);
+  const int pr = 4 * (vt >> 4), pc = 2 * (vt & 15);
+  const bool below = rank + 1 < s.cs && I + 1 < iend;   // the strip below is in the cluster
+  const float* lbk = a.LBblk + (int64_t)I * LEAF_BLOCKS * LEAF_BLOCK_FLOATS;
+  const int team = w >> 2;                            // 0 wavefront, 1 errors, 2 upper
+  // tiles of the strip above that we receive (in the cluster), n = 0 .. nin - 1
+  const int nin = live && rank > 0 && I >= 1 ? max(te - max(1, tb), 0) : 0;
+  constexpr uint32_t G_BYTES = TILE * KM * 4;
+  auto arm = [&](int n) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sh_u32(&S.gfull[n & 1])),
+                 "r"(G_BYTES)
+                 : "memory");
+  };
+  if (live && team == 1) {                            // read-only: before the wait
+    copy_block(&S.LBs[0][0], lbk, vt);
+    cp_async_commit();
+    if (vt < 36) S.LBs[TILE][vt] = 0.f;
+    if (vt < TILE) S.Xs[TILE][vt] = 0.f;
+  }
+  if (live && team == 2) {
+    copy_block(&S.LB1[0][0], lbk + LEAF_BLOCK_FLOATS, vt);
+    cp_async_commit();
+    if (vt == 0)
+      for (int n = 0; n < min(nin, 2); ++n) arm(n);
+  }
+  pdl_wait();
+  pdl_trigger();
+  stamp_begin(a.stamp);
+  if (live && team == 1) {
+    // -------------------------------------------------------- errors' team
+    float t1[4][2];
+    auto stage = [&](int tt) {
+      const int J = s.k + tt - I;
+      const int64_t c0 = (int64_t)J * TILE;
+      const float* lak = a.LAblk + (int64_t)J * LEAF_BLOCKS * LEAF_BLOCK_FLOATS;
+      copy_block(&S.LA0[tt & 1][0][0], lak, vt);
+      copy_block(&S.LA1[0][0], lak + LEAF_BLOCK_FLOATS, vt);
+      cp_async_commit();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) t1[i][0] = t1[i][1] = 0.f;
+      if (tt >= 2) {
+        auto fetch = [&](int d) {
+          const int b = d & 1;
+          copy_block(&S.B[b][2][0][0], lak + d * LEAF_BLOCK_FLOATS, vt);
+          const bool ve = J - d >= 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = vt + STRIP_TEAM * h, j = c / (TILE / 4), i4 = 4 * (c % (TILE / 4));
+            cp_async16(&S.B[b][0][j][i4],
+                       ve ? a.EtF + (c0 - (int64_t)TILE * d + j) * a.ldt + r0 + i4 : a.EtF, ve);
+          }
+          cp_async_commit();
+        };
+        fetch(2);
+        if (tt >= 3) fetch(3);
+#pragma unroll 1
+        for (int d = 2; d <= tt; ++d) {
+          if (d < tt) cp_async_wait_group<1>();
+          else cp_async_wait_group<0>();
+          team_sync<3>();
+          strip_product(S.B[d & 1][0], S.B[d & 1][2], pr, pc, t1);
+          if (d + 2 <= tt) {
+            team_sync<3>();   // buffer d & 1 is read
+            fetch(d + 2);
+          }
+        }
+      }
+      cp_async_wait_group<0>();
+      team_sync<3>();
+    };
+    stage(tb);
+    if (vt < TILE)
+      S.Lsub[vt] = make_float4(vt >= 1 ? S.LBs[vt][vt - 1] : 0.f, vt >= 2 ? S.LBs[vt][vt - 2] : 0.f,
+                               vt >= 3 ? S.LBs[vt][vt - 3] : 0.f, 0.f);
+    bool bad = false;
+    for (int tt = tb; tt <= te; ++tt) {
+      const int J = s.k + tt - I;
+      strip_sync();   // tile tt - 1 is rounded
+      float xr[LEAF_PER_THREAD];
+      uint32_t code[LEAF_PER_THREAD];
+      if (tt > tb) {
+        // the chain's rounding again, from its pre-rounding values: codes and errors
+        const int64_t c0 = (int64_t)(J - 1) * TILE;
+#pragma unroll
+        for (int i = 0; i < LEAF_PER_THREAD; ++i) {
+          const int e = vt + STRIP_TEAM * i, r = e / TILE, c = e % TILE;
+          const float x = S.Xd[r + c][c];
+          const float4 g = S.Srzl[r][c];
+          const float tc = fminf(fmaxf(fmaf(x, g.y, LEAF_R), g.z), g.w);
+          const bool real = (r0 + r) < a.m && (c0 + c) < a.n;
+          S.Es[c][r] = real ? fmaf(g.x, tc - LEAF_R, -x) : 0.f;
+          xr[i] = x;
+          code[i] = (uint32_t)(int)(tc - g.z);
+          bad |= !isfinite(x);
+        }
+      }
+      // the old grid has been read: the upper team may write the new one
+      asm volatile("bar.arrive 5, %0;" ::"n"(2 * STRIP_TEAM) : "memory");
+      if (tt > tb) team_sync<3>();
+      if (tt < te) {
+        if (tt > tb) strip_product(S.Es, S.LA1, pr, pc, t1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          S.T1s[pr + i][pc] = t1[i][0];
+          S.T1s[pr + i][pc + 1] = t1[i][1];
+        }
+        for (int e = vt; e < 4 * LEAF_ROWS_PADDED; e += STRIP_TEAM) (&S.Ebr[0][0])[e] = 0.f;
+      }
+      strip_sync();   // tile tt may be rounded
+      if (tt > tb) {
+        const int64_t c0 = (int64_t)(J - 1) * TILE;
+#pragma unroll
+        for (int i = 0; i < LEAF_PER_THREAD; ++i) {
+          const int e = vt + STRIP_TEAM * i, r = e / TILE, c = e % TILE;
+          a.X[(r0 + r) * a.ldx + c0 + c] = xr[i];
+          if ((r0 + r) < a.m && (c0 + c) < a.n) a.codes[(r0 + r) * a.n + c0 + c] = (uint8_t)code[i];
+          const float ev = S.Es[r][c];          // E^T row c0 + r, column r0 + c
+          const float hi = tf32_hi(ev);
+          const int64_t o = (c0 + r) * a.ldt + r0 + c;
+          a.EtH[o] = hi;
+          a.EtL[o] = ev - hi;
+          a.EtF[o] = ev;
+        }
+        team_sync<3>();   // the errors stand before a later window reads them
+      }
+      if (tt + 1 < te) stage(tt + 1);
+    }
+    if (bad) raise_status(a.status, BAKRON_ERR_NONFINITE);
+  } else if (live && team == 2) {
+    // ---------------------------------------------------------- upper team
+    float u[4][2], xv[4][2], sv[LEAF_PER_THREAD], iv[LEAF_PER_THREAD], zv[LEAF_PER_THREAD];
+    auto stage = [&](int tt) {
+      const int J = s.k + tt - I;
+      const int64_t c0 = (int64_t)J * TILE;
+#pragma unroll
+      for (int i = 0; i < LEAF_PER_THREAD; ++i) {
+        const int e = vt + STRIP_TEAM * i, p = e / TILE, c = e % TILE;
+        const bool real = (r0 + p) < a.m && (c0 + c) < a.n;
+        const int64_t og = real ? (r0 + p) * a.G + (c0 + c) / a.gsz : 0;
+        sv[i] = real ? a.scales[og] : 1.f;
+        zv[i] = real ? a.zeros[og] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < LEAF_PER_THREAD; ++i) iv[i] = 1.f / sv[i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 x2 = __ldcg(reinterpret_cast<const float2*>(a.X + (r0 + pr + i) * a.ldx + c0 + pc));
+        xv[i][0] = x2.x;
+        xv[i][1] = x2.y;
+        u[i][0] = u[i][1] = 0.f;
+      }
+      if (tt >= 2) {
+        // G[I-d, J], 2 <= d <= tt, was rounded at tt - d >= 0 by strip I - d
+        if (w == 8 && lane >= 2 && lane <= tt && I - lane >= s.ilo) flag_wait(s.fc, I - lane, J, a.status);
+        team_sync<4>();
+        auto fetch = [&](int d) {
+          const int b = d & 1;
+          copy_block(&S.B[b][3][0][0], lbk + d * LEAF_BLOCK_FLOATS, vt);
+          const bool vg = I - d >= 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = vt + STRIP_TEAM * h, j = c / (TILE / 4), i4 = 4 * (c % (TILE / 4));
+            cp_async16(&S.B[b][1][j][i4],
+                       vg ? a.Gout + (r0 - (int64_t)TILE * d + j) * a.ldx + c0 + i4 : a.Gout, vg);
+          }
+          cp_async_commit();
+        };
+        fetch(2);
+        if (tt >= 3) fetch(3);
+#pragma unroll 1
+        for (int d = 2; d <= tt; ++d) {
+          if (d < tt) cp_async_wait_group<1>();
+          else cp_async_wait_group<0>();
+          team_sync<4>();
+          strip_product(S.B[d & 1][3], S.B[d & 1][1], pr, pc, u);
+          if (d + 2 <= tt) {
+            team_sync<4>();   // buffer d & 1 is read
+            fetch(d + 2);
+          }
+        }
+      }
+      cp_async_wait_group<0>();
+      team_sync<4>();
+    };
+    stage(tb);
+    bool lost = false;   // a copy never came (the same for a whole warp)
+    for (int tt = tb; tt <= te; ++tt) {
+      const int J = s.k + tt - I;
+      const int64_t c0 = (int64_t)J * TILE;
+      strip_sync();   // tile tt - 1 is rounded
+      if (tt < te && tt >= 1 && I >= 1) {
+        // U's last term, from the G above, received as the n-th
+        const int n = tt - max(1, tb), b = n & 1;
+        if (rank > 0) {
+          if (!lost) lost = !strip_wait(&S.gfull[b], (uint32_t)(n >> 1) & 1u, s.fc.spin_cycles, a.status);
+        } else {
+          if (vt == 0) flag_wait(s.fc, I - 1, J, a.status);
+          team_sync<4>();
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = vt + STRIP_TEAM * h, j = c / (TILE / 4), i4 = 4 * (c % (TILE / 4));
+            cp_async16(&S.Gin[b][j][i4], a.Gout + (r0 - TILE + j) * a.ldx + c0 + i4, true);
+          }
+          cp_async_commit();
+          cp_async_wait_group<0>();
+          team_sync<4>();
+        }
+        strip_product(S.LB1, S.Gin[b], pr, pc, u);
+        if (rank > 0) {
+          team_sync<4>();
+          if (vt == 0) {
+            if (n + 2 < nin && !lost) arm(n + 2);
+            strip_arrive(&S.gfree[b], rank - 1);
+          }
+        }
+      }
+      asm volatile("bar.sync 5, %0;" ::"n"(2 * STRIP_TEAM) : "memory");   // the old grid has been read
+      if (tt < te) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          S.Xs[pr + i][pc] = xv[i][0] + u[i][0];
+          S.Xs[pr + i][pc + 1] = xv[i][1] + u[i][1];
+        }
+#pragma unroll
+        for (int i = 0; i < LEAF_PER_THREAD; ++i) {
+          const int e = vt + STRIP_TEAM * i;
+          S.Srzl[e / TILE][e % TILE] = make_float4(sv[i], iv[i], LEAF_R - zv[i],
+                                                   LEAF_R + (float)a.qmax - zv[i]);
+        }
+      }
+      strip_sync();   // tile tt may be rounded
+      if (tt + 1 < te) stage(tt + 1);
+    }
+  } else if (live && team == 0) {
+    // -------------------------------------------------------- wavefront team
+    for (int tt = tb; tt <= te; ++tt) {
+      const int J = s.k + tt - I;
+      const int64_t c0 = (int64_t)J * TILE;
+      strip_sync();   // tile tt - 1 is rounded
+      // its final G, which the team has stored, is published
+      if (t == STRIP_TEAM - 1 && tt > tb && tt < s.nb) {
+        __threadfence();
+        atomicExch(s.fc.done + (int64_t)I * s.fc.ntp + J - 1, 1u);
+      }
+      __syncwarp();
+      strip_sync();   // tile tt may be rounded
+      if (tt == te) break;
+      if (w == 0) {
+        wave_chain(S, S.LA0[tt & 1], r0, c0, a.m, a.n, a.clk);
+      } else {
+        const int g = w - 1, i0 = LEAF_ROWS_PER_HELPER * g;
+        const bool handed = tt + 1 < s.nb;     // a later tile of the block reads this G
+        const int n = tt - tb, b = n & 1;
+        if (handed && below && n >= 2)
+          strip_wait(&S.gfree[b], (uint32_t)((n >> 1) - 1) & 1u, s.fc.spin_cycles, a.status);
+        float Gg[LEAF_ROWS_PER_HELPER];
+        wave_helper<true>(S, S.LA0[tt & 1], g, lane, handed, Gg);
+        if (handed) {
+          if (below) {
+            // these rows as one copy into the strip below, counted on its barrier
+#pragma unroll
+            for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r) S.Gs[b][i0 + r][lane] = Gg[r];
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+              asm volatile(
+                  "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                      peer_u32(&S.Gin[b][i0][0], rank + 1)),
+                  "r"(sh_u32(&S.Gs[b][i0][0])), "r"((min(TILE, i0 + LEAF_ROWS_PER_HELPER) - i0) * KM * 4),
+                  "r"(peer_u32(&S.gfull[b], rank + 1))
+                  : "memory");
+          }
+#pragma unroll
+          for (int r = 0; r < LEAF_ROWS_PER_HELPER; ++r)
+            if (i0 + r < TILE) a.Gout[(r0 + i0 + r) * a.ldx + c0 + lane] = Gg[r];
+        }
+      }
+    }
+  }
+  // no CTA leaves while a neighbour may still write into its shared memory
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  stamp_end(a.stamp);
+}
+
+__global__ void __launch_bounds__(STRIP_THREADS, 1) k_strips(const __grid_constant__ LeafArgs a,
+                                                          const __grid_constant__ StripArgs s) {
+  strip_body(a, s);
+}
+
+// The same for H problems of one shape (LeafHeads): blockIdx.y = problem.
+__global__ void __launch_bounds__(STRIP_THREADS, 1) k_strips_heads(const __grid_constant__ LeafHeads L,
+                                                                const __grid_constant__ StripArgs s0) {
+  const int h = blockIdx.y;
+  const int64_t ds = (int64_t)h * L.slice;
+  LeafArgs a = L.base;
+  a.X = (float*)((char*)a.X + ds);
+  a.EtH = (float*)((char*)a.EtH + ds);
+  a.EtL = (float*)((char*)a.EtL + ds);
+  a.EtF = (float*)((char*)a.EtF + ds);
+  a.Gout = (float*)((char*)a.Gout + ds);
+  a.status = (int*)((char*)a.status + ds);
+  a.LBblk = L.LBblk[h];
+  a.LAblk = L.LAblk[h];
+  a.codes = L.codes[h];
+  a.scales = L.scales[h];
+  a.zeros = L.zeros[h];
+  StripArgs s = s0;
+  s.fc.done = (unsigned*)((char*)s.fc.done + ds);
+  s.claim = (unsigned*)((char*)s.claim + ds);
+  strip_body(a, s);
 }
 
 // A whole block of leaves [k, l) in one launch (LEAF_FLOW).  The block's
@@ -1403,6 +1905,103 @@ static void leaf(SolveArgs& a, int K, int window) {
   note(a, launch_leaf_window(window, grid, block, sm, a.s, K, la));
 }
 
+// CTAs of k_strips that run at once in clusters of 1 << log_cs, on the current
+// device (queried once per device); 0 if that cannot be told.
+static int strip_capacity(int log_cs) {
+  static std::mutex mu;
+  static int cap[64][4];
+  static bool done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!done[dev]) {
+    for (int i = 0; i < 4; ++i) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(1u << i);
+      cfg.blockDim = dim3(STRIP_THREADS);
+      cfg.dynamicSmemBytes = sizeof(StripSmem);
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 1u << i;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_strips, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+      cap[dev][i] = n << i;
+    }
+    done[dev] = true;
+  }
+  return cap[dev][log_cs];
+}
+
+// Block [k, l) of H problems as one launch of strips: their count, and the CTAs of a
+// cluster, the largest power of two (at most STRIP_CLUSTER) that they fill and of
+// which all run at once.  False if there is none: strips that wait for others to
+// finish the whole block would cost more than a launch per anti-diagonal, whose
+// CTAs share an SM (two of k_leaf, one of k_strips).
+static bool strip_args(const SolveArgs& a, int k, int l, int H, StripArgs& s) {
+  s.k = k;
+  s.nb = l - k;
+  s.ilo = max(0, k - (a.Nt - 1));
+  s.nstrips = min(l - 1, a.Mt - 1) - s.ilo + 1;
+  s.fc = FlowCtx{a.flow_done, a.ntp, a.spin_cycles};
+  s.claim = a.flow_claim + k;
+  static_assert(STRIP_CLUSTER == 8, "clusters of 1, 2, 4, 8");
+  for (int i = 3; i >= 0; --i) {
+    s.cs = 1 << i;
+    if (i > 0 && s.cs / 2 >= s.nstrips) continue;
+    if (ceil_div(s.nstrips, s.cs) * s.cs * H <= strip_capacity(i)) return true;
+  }
+  return false;
+}
+
+// Flops of a block's leaves: the in-tile feedback and the window's products, 2 *
+// 32^3 each, per tile.
+static double strip_flops(const SolveArgs& a, int k, int l) {
+  double f = 0.0;
+  for (int K = k; K < l; ++K)
+    f += 2.0 * TILE * TILE * TILE * (1 + window_products(K - k)) *
+         (min(K, a.Mt - 1) - max(0, K - (a.Nt - 1)) + 1);
+  return f;
+}
+
+// Clusters of s.cs CTAs along x, with programmatic dependent launch.
+template <typename K, typename A>
+static cudaError_t launch_strips(K kernel, const A& args, const StripArgs& s, int heads, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ceil_div(s.nstrips, s.cs) * s.cs), (unsigned)heads);
+  cfg.blockDim = dim3(STRIP_THREADS);
+  cfg.dynamicSmemBytes = sizeof(StripSmem);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)s.cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, args, s);
+}
+
+static void leaf_block(SolveArgs& a, int k, int l) {
+  StripArgs s;
+  if (!strip_args(a, k, l, 1, s)) {
+    for (int K = k; K < l; ++K) leaf(a, K, K - k);
+    return;
+  }
+  LaunchScope ls(kFamLeaf, a.s, strip_flops(a, k, l));
+  LeafArgs la = a.la;
+  la.stamp = ls.stamp();
+  note(a, launch_strips(k_strips, la, s, 1, a.s));
+}
+
 // Dynamic shared memory of the leaf and subtree kernels above the 48 KB
 // default, set once per process.
 static cudaError_t ensure_leaf_attrs() {
@@ -1412,6 +2011,12 @@ static cudaError_t ensure_leaf_attrs() {
   if (done) return cudaSuccess;
   const int sm = (int)sizeof(LeafSmem), ss = (int)sizeof(SubtreeSmem);
   cudaError_t e = set_leaf_smem<0>(sm);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(StripSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_strips_heads, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(StripSmem));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_subtree, cudaFuncAttributeMaxDynamicSharedMemorySize, ss);
   if (e == cudaSuccess)
@@ -1576,7 +2181,7 @@ static void rec(SolveArgs& a, int k, int l) {
   if (l - k <= a.leaf_block) {
     // a block of leaves: leaf K applies what anti-diagonals k .. K-1 send it
     // (the Alg. 5 nodes inside [k, l)), so no band launch is needed here
-    for (int K = k; K < l; ++K) leaf(a, K, K - k);
+    leaf_block(a, k, l);
     return;
   }
   if (l - k <= a.subtree_max && a.subtree_grid > 0) {
@@ -1687,11 +2292,9 @@ int solve_impl(const void* W, int wdt, int m, int n, int64_t ldw, const void* fa
     if (rc != BAKRON_OK) return rc;
   }
   reset_launch_count();
-  if (keep_status)
-    BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_status + 64, 0, 256 - 64, s));
-  else
-    BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_status, 0, 256, s));
-  if (a.leaf_flow) BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_flow, 0, sl.flow_bytes, s));
+  // the status word, the grid-barrier words and the tiles' flags after them
+  const size_t keep = keep_status ? 64 : 0;
+  BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_status + keep, 0, sl.off_X - sl.off_status - keep, s));
   if (!grid_given) launch_grid(W, wdt, m, n, ldw, a.gsz, a.G, a.qmax, scales, zeros, s);
   {
     const int rc = launch_init(W, wdt, m, n, ldw, a.X, a.mp, a.np, s);
@@ -1742,6 +2345,15 @@ void heads_rec(HeadsRun& r, int k, int l) {
   const SolveArgs& a0 = r.a[0];
   if (l - k <= a0.leaf_block) {
     heads_join(r);
+    StripArgs s;
+    if (strip_args(a0, k, l, r.H, s)) {
+      LaunchScope ls(kFamLeaf, r.main, strip_flops(a0, k, l) * r.H);
+      LeafHeads lh = r.lh;
+      lh.base.stamp = ls.stamp();
+      const cudaError_t e = launch_strips(k_strips_heads, lh, s, r.H, r.main);
+      if (e != cudaSuccess) r.rc = cuda_fail(e, __FILE__, __LINE__);
+      return;
+    }
     for (int K = k; K < l; ++K) {
       const int ilo = max(0, K - (a0.Nt - 1)), ihi = min(K, a0.Mt - 1);
       LaunchScope ls(kFamLeaf, r.main, 2.0 * TILE * TILE * TILE * (1 + window_products(K - k)) *
@@ -1824,7 +2436,7 @@ int solve_heads_impl(int H, const void* const* W, int wdt, int m, int n, int64_t
   // status word), the grid, X from W
   for (int h = 0; h < H; ++h) {
     char* ws = workspace + (size_t)h * slice;
-    BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_status + 64, 0, 256 - 64, lanes[h]));
+    BK_CUDA_OK(cudaMemsetAsync(ws + sl.off_status + 64, 0, sl.off_X - sl.off_status - 64, lanes[h]));
     launch_grid(W[h], wdt, m, n, ldw, a[h].gsz, a[h].G, a[h].qmax, scales[h], zeros[h], lanes[h]);
     const int rc = launch_init(W[h], wdt, m, n, ldw, a[h].X, a[h].mp, a[h].np, lanes[h]);
     if (rc != BAKRON_OK) r.rc = rc;
