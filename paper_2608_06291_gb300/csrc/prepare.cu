@@ -218,8 +218,8 @@ struct PotrfSmem {
   int2 xs[PH][PH + 1];           // columns of X11, then rows of X22 (split)
   int2 ts[PH][PH + 1];           // L21, then columns of L21 X11 (split)
   int ec[PH], er[PH], et[PH];
-  double pub[8][8];
-  double rinv[NB];
+  double col[8][NB];             // their entries as each became the pivot column
+  double rinv[NB], diag[NB];
 };
 
 __device__ __forceinline__ void workers_sync() {
@@ -232,6 +232,14 @@ __device__ __forceinline__ double rsqrt64(double p) {
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
   const double e = fma(-p * r, r, 1.0);
   return fma(r * e, fma(0.375, e, 0.5), r);
+}
+
+// 1 / p the same way.
+__device__ __forceinline__ double rcp64(double p) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+  const double e = fma(-p, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 
 // An exponent above three times the largest magnitude of a warp's values (32
@@ -248,12 +256,14 @@ __device__ __forceinline__ int warp_exp8(double x) {
 //
 // The fp64 units take a warp's instruction every 64 cycles per scheduler, so
 // the count of those sets the time, and what can be is done in integers.  Eight
-// columns at a time: a thread per row with the columns' entries in registers, fp64
-// (the unscaled pivot and the eight rows it shares are published once per column,
-// 1 / sqrt is formed redundantly; about 1000 cycles a column, 1700 with both
-// halves' rows in one warp); then one update of the rest by all warps on split
-// 56-bit values (three 32 x 32 + 64 multiply-adds each).  The inverse by halving:
-// 8 x 8 blocks and the first two levels in fp64, the last in integers.
+// columns at a time in fp64: four warps, two threads a row with every other column
+// in registers; per column the entries are published, and a row's entry over the
+// pivot (a reciprocal) times the eight rows' entries updates what it holds, so that
+// the square roots wait for the end, a lane each (6 fp64 instructions a column; a
+// thread per row with 1 / sqrt inside each column took 10).  Then one update of the
+// rest by all warps on split 56-bit values (three 32 x 32 + 64 multiply-adds each).
+// The inverse by halving: 8 x 8 blocks and the first two levels in fp64, the last
+// in integers.
 __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // this thread's entries of a lower triangle of up to 63 rows, row by row
@@ -277,38 +287,46 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
   }
   workers_sync();
   for (int c0 = 0; c0 < NB; c0 += 8) {
-    if (t < NB && t >= (c0 & 32)) {   // whole warps: rows of finished warps are done
-      const int r = t;
-      const int live = NB - (c0 & 32);
-      double a[8];
+    // thread (row r, half hc): columns c0 + hc, + 2, + 4, + 6; a warp whose rows are
+    // all done stays away
+    if (t < 2 * NB && (t & (NB - 1)) >= (c0 & 32)) {
+      const int r = t & (NB - 1), hc = t / NB, live = 2 * (NB - (c0 & 32));
+      double a[4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) a[j] = r >= c0 ? M.cur[r][j] : 0.0;
+      for (int i = 0; i < 4; ++i) a[i] = r >= c0 ? M.cur[r][2 * i + hc] : 0.0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        if (r >= c0 && r < c0 + 8) M.pub[j][r - c0] = a[j];
+        if (hc == (j & 1)) M.col[j][r] = a[j / 2];
         asm volatile("bar.sync 2, %0;" ::"r"(live) : "memory");
-        double p = M.pub[j][j];
+        if (j == 7) break;
+        double p = M.col[j][c0 + j];
+        if (!(p > 0.0)) p = 1.0;
+        const double lr = M.col[j][r] * rcp64(p);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (2 * i + hc > j) a[i] = fma(-lr, M.col[j][c0 + 2 * i + hc], a[i]);
+      }
+      if (hc == 0 && r >= c0 && r < c0 + 8) {   // a pivot per lane
+        double p = M.col[r - c0][r];
         if (!(p > 0.0)) {
-          if (r == c0 + j) raise_status(status, BAKRON_ERR_NOT_SPD);
+          raise_status(status, BAKRON_ERR_NOT_SPD);
           p = 1.0;
         }
         const double ri = rsqrt64(p);
-        const double l = (r == c0 + j ? p : a[j]) * ri, lr = l * ri;
-        a[j] = l;
-        if (r == c0 + j) {
-          M.rinv[r] = ri;
-          S.ldiag[k0 + r] = l;
-        }
-#pragma unroll
-        for (int k = j + 1; k < 8; ++k) a[k] = fma(-lr, M.pub[j][k], a[k]);
+        M.rinv[r] = ri;
+        M.diag[r] = p * ri;
+        S.ldiag[k0 + r] = p * ri;
       }
+      asm volatile("bar.sync 2, %0;" ::"r"(live) : "memory");
       if (r >= c0) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const long long v = c0 + j <= r ? to_fix(a[j], 63) : 0;
+        for (int i = 0; i < 4; ++i) {
+          const int j = 2 * i + hc;
+          const double l = r == c0 + j ? M.diag[r] : a[i] * M.rinv[c0 + j];
+          const long long v = c0 + j <= r ? to_fix(l, 63) : 0;
           if (c0 + j <= r) M.a[r][c0 + j] = v;
           M.l8[r][j] = split56(v);
-          M.inv[r][c0 + j] = a[j];       // the factor in fp64, for the halving
+          M.inv[r][c0 + j] = l;            // the factor in fp64, for the halving
         }
       }
     }
