@@ -75,8 +75,7 @@ __global__ void k_grid(const void* W, int wdt, int m, int n, int64_t ldw, int gs
 // only move a value lying within rounding of a midpoint between two levels
 // to the other level, where both have the same squared error.  An all-zero row/group uses amax = 1.  Stored in
 // the affine form the solve reads: z = l, codes 0..2l.  One block of
-// GRID_SYM_THREADS per (row, group); the row is re-read from L1 per
-// candidate; sums are fp32 per thread, then a fixed tree.
+// GRID_SYM_THREADS per (row, group); sums are fp32 per thread, then a fixed tree.
 constexpr int GRID_SYM_THREADS = 256;
 
 __device__ __forceinline__ float block_sum_or_max(float v, bool is_max, float* red) {
@@ -93,10 +92,39 @@ __device__ __forceinline__ float block_sum_or_max(float v, bool is_max, float* r
   return v;
 }
 
+// SYM_GROUP sums at once, each reduced in block_sum_or_max's order.
+constexpr int SYM_GROUP = 4;
+__device__ __forceinline__ void block_sums(float (&v)[SYM_GROUP], float (*red)[SYM_GROUP]) {
+  for (int o = 16; o; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < SYM_GROUP; ++j) v[j] = v[j] + __shfl_xor_sync(0xffffffffu, v[j], o);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();                       // red[] free from the last call
+  if (lane == 0) {
+#pragma unroll
+    for (int j = 0; j < SYM_GROUP; ++j) red[warp][j] = v[j];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < SYM_GROUP; ++j) {
+    v[j] = red[0][j];
+    for (int w = 1; w < GRID_SYM_THREADS / 32; ++w) v[j] = v[j] + red[w][j];
+  }
+}
+
+// NV > 0: the row/group has at most NV * GRID_SYM_THREADS values, which a thread
+// keeps in registers (zeros past the end: a zero adds nothing to any candidate's
+// error) and scores against SYM_GROUP candidates per reduction; NV = 0: any length,
+// read again per candidate.  Same sums in the same order either way.  2048 x 4096
+// bf16, 51 candidates: re-reading and converting every value per candidate and one
+// reduction (two barriers) each took 0.19 ms.
+template <int NV>
 __global__ void __launch_bounds__(GRID_SYM_THREADS)
     k_grid_sym(const void* W, int wdt, int m, int n, int64_t ldw, int gsz, int G, int levels,
                int K, float* scales, float* zeros) {
   __shared__ float red[GRID_SYM_THREADS / 32];
+  __shared__ float reds[GRID_SYM_THREADS / 32][SYM_GROUP];
   const int64_t items = (int64_t)m * G;
   // block-uniform loop: every thread of a block reaches the same barriers
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
@@ -106,25 +134,59 @@ __global__ void __launch_bounds__(GRID_SYM_THREADS)
       return (wdt == BAKRON_BF16) ? __bfloat162float(((const __nv_bfloat16*)W)[base + c])
                                   : ((const float*)W)[base + c];
     };
-    float amax = 0.f;
-    for (int c = threadIdx.x; c < gsz; c += GRID_SYM_THREADS) amax = fmaxf(amax, fabsf(load(c)));
-    amax = block_sum_or_max(amax, true, red);
-    if (amax == 0.f) amax = 1.f;
-    const float L = (float)levels;
-    float best_s = 0.f, best_err = INFINITY;
-    for (int k = 0; k <= K; ++k) {
-      const float t = K == 0 ? __fdiv_rn(1.f, L)
+    auto scale = [&](int k, float amax) -> float {
+      const float t = K == 0 ? __fdiv_rn(1.f, (float)levels)
                              : __fdiv_rn((float)(2 * K - k), (float)(2 * K * levels));
-      const float s = __fmul_rn(amax, t), rs = __fdiv_rn(1.f, s);
-      float err = 0.f;
-      for (int c = threadIdx.x; c < gsz; c += GRID_SYM_THREADS) {
-        const float v = load(c);
-        const float q = fminf(fmaxf(rintf(v * rs), -L), L);
-        const float d = fmaf(s, q, -v);
-        err = fmaf(d, d, err);
+      return __fmul_rn(amax, t);
+    };
+    const float L = (float)levels;
+    auto add = [&](float v, float s, float rs, float err) -> float {
+      const float q = fminf(fmaxf(rintf(v * rs), -L), L);
+      const float d = fmaf(s, q, -v);
+      return fmaf(d, d, err);
+    };
+    float best_s = 0.f, best_err = INFINITY, amax = 0.f;
+    if constexpr (NV > 0) {
+      float v[NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int c = threadIdx.x + GRID_SYM_THREADS * i;
+        v[i] = c < gsz ? load(c) : 0.f;
+        amax = fmaxf(amax, fabsf(v[i]));
       }
-      err = block_sum_or_max(err, false, red);
-      if (k == 0 || err < best_err) { best_err = err; best_s = s; }
+      amax = block_sum_or_max(amax, true, red);
+      if (amax == 0.f) amax = 1.f;
+      for (int k0 = 0; k0 <= K; k0 += SYM_GROUP) {
+        float s[SYM_GROUP], rs[SYM_GROUP], err[SYM_GROUP];
+#pragma unroll
+        for (int j = 0; j < SYM_GROUP; ++j) {
+          s[j] = scale(min(k0 + j, K), amax);
+          rs[j] = __fdiv_rn(1.f, s[j]);
+          err[j] = 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+#pragma unroll
+          for (int j = 0; j < SYM_GROUP; ++j) err[j] = add(v[i], s[j], rs[j], err[j]);
+        block_sums(err, reds);
+#pragma unroll
+        for (int j = 0; j < SYM_GROUP; ++j)
+          if (k0 + j <= K && (k0 + j == 0 || err[j] < best_err)) {
+            best_err = err[j];
+            best_s = s[j];
+          }
+      }
+    } else {
+      for (int c = threadIdx.x; c < gsz; c += GRID_SYM_THREADS) amax = fmaxf(amax, fabsf(load(c)));
+      amax = block_sum_or_max(amax, true, red);
+      if (amax == 0.f) amax = 1.f;
+      for (int k = 0; k <= K; ++k) {
+        const float s = scale(k, amax), rs = __fdiv_rn(1.f, s);
+        float err = 0.f;
+        for (int c = threadIdx.x; c < gsz; c += GRID_SYM_THREADS) err = add(load(c), s, rs, err);
+        err = block_sum_or_max(err, false, red);
+        if (k == 0 || err < best_err) { best_err = err; best_s = s; }
+      }
     }
     if (threadIdx.x == 0) {
       scales[item] = best_s;
@@ -139,8 +201,11 @@ int launch_grid_sym(const void* W, int wdt, int m, int n, int64_t ldw, int level
   const int gsz = group_size == 0 ? n : group_size;
   const int G = n / gsz;
   const int64_t blocks = std::min<int64_t>((int64_t)m * G, 152 * 16);
-  k_grid_sym<<<(unsigned)blocks, GRID_SYM_THREADS, 0, s>>>(
-      W, wdt, m, n, ldw, gsz, G, levels, shrink_steps, scales, zeros);
+  const int per = ceil_div(gsz, GRID_SYM_THREADS);     // values of a thread
+  const auto kernel = per <= 1 ? k_grid_sym<1> : per <= 4 ? k_grid_sym<4> : per <= 16 ? k_grid_sym<16>
+                      : per <= 32 ? k_grid_sym<32> : k_grid_sym<0>;
+  kernel<<<(unsigned)blocks, GRID_SYM_THREADS, 0, s>>>(W, wdt, m, n, ldw, gsz, G, levels,
+                                                       shrink_steps, scales, zeros);
   BK_CUDA_OK(cudaGetLastError());
   return BAKRON_OK;
 }
