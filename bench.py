@@ -154,7 +154,7 @@ def host_info() -> dict:
 # The sources that define the solve's kernels and its launch schedule: the
 # DRAM figures in profiles/traffic.txt stand while these are unchanged.
 SOLVE_SOURCES = ("common.cuh", "profile.cu", "profile.cuh", "solve.cu", "solve.cuh",
-                 "tc_gemm.cu", "tc_gemm.cuh", "tune.cu", "tune.cuh")
+                 "tc_gemm.cu", "tc_gemm.cuh", "tcgen05.cuh", "tune.cu", "tune.cuh")
 
 
 def _csrc_hash():
@@ -528,7 +528,7 @@ def run_gpu(args):
     step_ns = cyc / mhz * 1e3
     floor_ms = (m + n - 1) * step_ns * 1e-6
     tile_steps = leaf_n * (2 * TILE - 1)
-    leaf_roof = {"kernel": "k_leaf: 32 x 32 tiles, one CTA each, wavefront of 63 in-tile steps",
+    leaf_roof = {"kernel": "k_strips: 32 x 32 tiles, one CTA per 32-row strip, wavefront of 63 in-tile steps per tile",
                  "bound": "latency", "achieved": (m + n - 1) / (leaf_ms / 1e3),
                  "peak": 1e9 / step_ns, "unit": "element anti-diagonals/s",
                  "frac": floor_ms / leaf_ms if leaf_ms > 0 else None,

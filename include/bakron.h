@@ -256,8 +256,9 @@ int bakron_sample_sqnorms(const void* Y, int ydtype, int k, int d, int64_t ldy,
  *            lanes fork from `stream` and join back into it through events,
  *            so later work on `stream` sees every result.  With S = H >= 2
  *            (one lane per problem) the leaves of all problems share one
- *            launch per tile anti-diagonal and each tensor-core band stage
- *            one launch, on `stream` itself (unless the shape's schedule
+ *            launch per block of tile anti-diagonals (or one per anti-diagonal,
+ *            where a block's strips do not all run at once) and each
+ *            tensor-core band stage one launch, on `stream` itself (unless the shape's schedule
  *            uses dataflow leaves or persistent subtrees)
  *   workspace device, >= bakron_batched_workspace_bytes(m, n, min(S, H))
  *            bytes: lane l uses slice l (bakron_workspace_bytes(m, n) rounded

@@ -9,7 +9,7 @@
 // is enqueued on lane h mod S of S library-owned streams, which fork from the
 // caller's stream through an event and join back into it through one event
 // per lane.  With one lane per problem (S = H), the leaves of all problems
-// share one launch per tile anti-diagonal on the caller's stream, and so do
+// share one launch per block of tile anti-diagonals on the caller's stream, and so do
 // the tensor-core band stages (one launch per stage, blockIdx.z = problem);
 // only CUDA-core band products of narrow nodes run per problem on the lanes
 // (solve_heads_impl).  Each lane owns one slice of the workspace and runs its problems

@@ -21,8 +21,8 @@ int solve_impl(const void* W, int wdt, int m, int n, int64_t ldw, const void* fa
                bool keep_status);
 
 // H <= 32 problems of one shape solved side by side, problem h in the
-// workspace slice `slice` bytes after problem h - 1's: each tile anti-diagonal's
-// leaves of all problems in one launch on `main`, each node's tensor-core band
+// workspace slice `slice` bytes after problem h - 1's: each block's leaves of all
+// problems in one launch on `main` (or one per tile anti-diagonal), each node's tensor-core band
 // stages of all problems in one launch each on `main`, a narrower node's
 // CUDA-core band products per problem on lanes[h]; the lanes must have been
 // forked from `main` (an event recorded on main and waited on by every
