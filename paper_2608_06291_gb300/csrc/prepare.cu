@@ -30,7 +30,11 @@
 //     8 bits apart, is formed in 64-bit integers modulo 2^64: it cannot be lost,
 //     since the result itself is known to fit (Cauchy-Schwarz).  Dropped digit
 //     products are below 2^-53 of the product of the norms.
-// Diagonal 64 x 64 blocks are factored and inverted in fp64 by one CTA.
+// Diagonal 64 x 64 blocks are factored and inverted by one CTA, in fp64 and 56-bit
+// integers.
+//
+// Measured on GB300, both sides 4096: 160.2 ms with the products on the fp64 units,
+// 9.3 so; 1531 + 1000: 26.7 -> 2.7.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -461,6 +465,12 @@ __global__ void __launch_bounds__(WT) k_prep_first(const PrepArgs P) {
 //            with the other tiles
 //   OZ_INV1  node (i0, h) of the inverse: R = X11^T L21^T, above C's diagonal
 //   OZ_INV2  X21 = -X22 R^T
+// 128 x 128 tiles and 64-deep chunks, because the fourteen digit planes of one chunk
+// just fit shared memory.  What bounds a chunk: cutting the operands (6 to 9 thousand
+// cycles, integer work and the loads' latency), then 112 MMAs of 62 cycles and the
+// sums, which partly run beside them (12 thousand); nothing of the next chunk can
+// start meanwhile.  9 to 10 us, against 20 to 28 with shifts by run-time counts and
+// a warp of its own for the MMAs.
 enum OzMode { OZ_TRSM, OZ_SYRK, OZ_INV1, OZ_INV2 };
 
 // Seven digits of eight values (Q63) to the planes: 16 bytes of a row each, in

@@ -527,8 +527,8 @@ __device__ __forceinline__ void wave_chain(SM& S, const float (*LA0)[KM], int64_
   // L1_1 (left neighbour, last step, still in flight from its shuffle) are
   // new; the sum of the older ones is formed first so that these two enter
   // last.  The shuffles the next step needs are issued as soon as their
-  // inputs exist.  Entries off the tile or outside W get a zero error (the
-  // factor mk).
+  // inputs exist.  Entries off the tile or outside W get a zero
+  // error.
   auto step = [&](int d, bool odd, float pre, const float4& g, const float4& lb) {
     const int p = d - q;
     float A = fmaf(la2, L2_2, pre);
