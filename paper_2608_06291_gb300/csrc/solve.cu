@@ -1138,18 +1138,17 @@ __device__ __forceinline__ void strip_body(const LeafArgs& a, const StripArgs& s
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sh_u32(&S.gfree[b])), "r"(1));
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (rank == 0) {
-      // clusters take their strips in the order they start, so the strips above
-      // are held by clusters that run or have run
-      const unsigned c = atomicAdd(s.claim, 1u);
-      for (int r = 0; r < s.cs; ++r)
-        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(peer_u32(&S.claim, r)), "r"(c)
-                     : "memory");
-    }
+    // clusters take their strips in the order they start, so the strips above
+    // are held by clusters that run or have run
+    if (rank == 0) S.claim = (int)atomicAdd(s.claim, 1u);
   }
   __syncthreads();
+  // every CTA of the cluster has begun and its barriers stand: only now may their
+  // shared memory be touched from outside
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-  const int I = s.ilo + S.claim * s.cs + rank, iend = s.ilo + s.nstrips;
+  int claim;
+  asm volatile("ld.relaxed.cluster.shared::cluster.s32 %0, [%1];" : "=r"(claim) : "r"(peer_u32(&S.claim, 0)) : "memory");
+  const int I = s.ilo + claim * s.cs + rank, iend = s.ilo + s.nstrips;
   const int64_t r0 = (int64_t)I * TILE;
   const int tb = max(0, I - s.k), te = I < iend ? min(s.nb, a.Nt + I - s.k) : tb;   // tiles t in [tb, te)
   const bool live = te > tb;
