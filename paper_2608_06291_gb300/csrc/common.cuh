@@ -125,6 +125,25 @@ struct PrepareLayout {
   }
 };
 
+// Where prepare keeps its matrices: per side C (dp x dp 8-byte words) in the factor
+// planes that the assembly writes last, the small arrays in the leaf blocks (written
+// after that), X in the workspace.  Its loads are 32 bytes wide, while a caller's
+// buffers need only suit their own element types, so everything sits on the next
+// 32-byte boundary: both C up by the same bytes (the last ones in rB, which is
+// written after C has been read), the rest into room that is there.
+struct PrepareScratch {
+  char *CA, *CB, *smallA, *smallB, *XA, *XB;
+  PrepareScratch(const FactorLayout& fl, const PrepareLayout& pl, char* factors, char* workspace) {
+    char* f = factors + (-(uintptr_t)factors & 31);
+    CA = f + fl.off_LAH;
+    CB = f + fl.off_LBH;
+    smallA = f + fl.off_LAblk;
+    smallB = f + fl.off_LBblk;
+    XA = workspace + pl.off_X + (-(uintptr_t)workspace & 31);
+    XB = XA + size_t(fl.np * fl.np) * 8;
+  }
+};
+
 // Programmatic dependent launch.  Every kernel of the solve waits for the
 // previous kernel on the stream to complete (pdl_wait) before it touches data
 // that kernel or its predecessors wrote, and only then lets the next kernel

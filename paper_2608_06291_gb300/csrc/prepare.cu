@@ -1024,15 +1024,13 @@ cudaError_t prep_attrs() {
   return e;
 }
 
-// Where one side keeps its matrices: C in the factor planes that the assembly
-// writes last, small arrays in the leaf blocks (written after that), X in the
-// workspace.
-PrepSide make_side(const float* H, int d, int64_t dp, char* planes, char* scratch, char* x) {
+// One side from where its matrices are (PrepareScratch).
+PrepSide make_side(const float* H, int d, int64_t dp, char* c, char* scratch, char* x) {
   PrepSide S;
   S.H = H;
   S.d = d;
   S.dp = (int)dp;
-  S.C = (long long*)planes;
+  S.C = (long long*)c;
   S.X = (double*)x;
   S.dinv = (double*)scratch;
   S.ldiag = S.dinv + dp * NB;
@@ -1044,7 +1042,8 @@ PrepSide make_side(const float* H, int d, int64_t dp, char* planes, char* scratc
   S.tr = S.xr + dp;
   return S;
 }
-// bytes of `scratch` per row of a side: 64 + 1 fp64, five ints (and the mean)
+// bytes of `scratch` per row of a side: 64 + 1 fp64, five ints (and the mean, and the
+// shift to a 32-byte boundary)
 static_assert((NB + 1) * 8 + 5 * 4 + 16 <= LEAF_BLOCKS * LEAF_BLOCK_FLOATS * 4 / TILE, "scratch fits the leaf blocks");
 
 }  // namespace
@@ -1058,9 +1057,9 @@ int prepare_impl(const float* A, const float* B, int m, int n, float damp, void*
   BK_CUDA_OK(prep_attrs());
   BK_CUDA_OK(cudaMemsetAsync(ws + pl.off_status, 0, 256, s));
   PrepArgs P;
-  P.side[0] = make_side(A, n, fl.np, f + fl.off_LAH, f + fl.off_LAblk, ws + pl.off_X);
-  P.side[1] = make_side(B, m, fl.mp, f + fl.off_LBH, f + fl.off_LBblk,
-                        ws + pl.off_X + (size_t)(fl.np * fl.np) * 8);
+  const PrepareScratch at(fl, pl, f, ws);
+  P.side[0] = make_side(A, n, fl.np, at.CA, at.smallA, at.XA);
+  P.side[1] = make_side(B, m, fl.mp, at.CB, at.smallB, at.XB);
   P.damp = damp;
   P.status = (int*)(ws + pl.off_status);
   P.spin_cycles = spin_cycles_from_env();
