@@ -27,9 +27,16 @@
 //     each an fp16 integer of [-128, 127].  The 28 products of digit planes (i, j) with
 //     i + j <= 6 are exact in the tensor cores' fp32 accumulators over 64 terms
 //     (7 * 64 * 2^14 < 2^23); planes of equal i + j share one.  Their sum, shifted
-//     8 bits apart, is formed in 64-bit integers modulo 2^64: it cannot be lost,
-//     since the result itself is known to fit (Cauchy-Schwarz).  Dropped digit
-//     products are below 2^-53 of the product of the norms.
+//     8 bits apart, is formed in 64-bit integers modulo 2^64, which is right where
+//     the result itself fits.  Dropped digit products are below 2^-53 of the product
+//     of the norms.
+//   * Of a positive definite matrix every result fits: entries of the factor and of
+//     the Schur complements, and sums over a factor's rows, are below 0.976
+//     (Cauchy-Schwarz).  Of another it need not, and a wrapped pivot could look
+//     positive.  So each step raises NOT_SPD where its own result does not fit: the
+//     sums of a panel's products by their leading digits (OZ_FIT), a factor's entries
+//     by their size, a Schur complement by its subtraction's overflow and by a
+//     diagonal that is not positive.  Nothing that wrapped is used unnoticed.
 // Diagonal 64 x 64 blocks are factored and inverted by one CTA, in fp64 and 56-bit
 // integers.
 //
@@ -218,7 +225,8 @@ struct PotrfSmem {
   long long a[NB][NB + 1];       // Q63: the block, then its factor
   double inv[NB][NB + 1];        // the inverse; above the diagonal, products of its halving
   double cur[NB][9];             // the eight columns being factored
-  __align__(16) int2 l8[NB][10]; // the same, factored, split (rows of 80 bytes: no conflicts)
+  __align__(16) int2 l8[2][NB][10]; // the same, factored, split (rows of 80 bytes: no conflicts);
+                                    // by the parity of the eight
   int2 xs[PH][PH + 1];           // columns of X11, then rows of X22 (split)
   int2 ts[PH][PH + 1];           // L21, then columns of L21 X11 (split)
   int ec[PH], er[PH], et[PH];
@@ -256,7 +264,7 @@ __device__ __forceinline__ int warp_exp8(double x) {
 // Factors the block of C at (k0, k0) and inverts the factor, by all WT threads
 // of the CTA.  Writes the factor to C, its inverse to dinv and to X's diagonal
 // block, the exponents of the inverse's rows to f.  A pivot that is not positive
-// raises NOT_SPD and is replaced by 1.
+// raises NOT_SPD and is replaced by 1; so does anything that does not fit.
 //
 // The fp64 units take a warp's instruction every 64 cycles per scheduler, so
 // the count of those sets the time, and what can be is done in integers.  Eight
@@ -270,6 +278,7 @@ __device__ __forceinline__ int warp_exp8(double x) {
 // in integers.
 __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  bool bad = false;
   // this thread's entries of a lower triangle of up to 63 rows, row by row
   constexpr int TRI = ((NB - 8) * (NB - 7) / 2 + WT - 1) / WT;
   int tr[TRI], tc[TRI];
@@ -290,7 +299,25 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
     if (c < 8) M.cur[r][c] = from_fix(v, -63);
   }
   workers_sync();
+  // Whether row r of the eight columns from c on, and the update by them, fit: entries
+  // below one, their norm too (0.99, to 2^-11), and a positive diagonal left.
+  auto fits = [&](int r, int c, bool diagonal) {
+    const int2* l = M.l8[(c >> 3) & 1][r];
+    unsigned norm = 0;                                  // unit 2^-28
+    bool ok = !diagonal || M.a[r][r] > 0;
+    for (int j = 0; j < 8; ++j) {
+      if (c + j > r) break;
+      ok &= (__double2hiint(M.inv[r][c + j]) & 0x7fffffff) < 0x3ff00000;
+      const int l14 = l[j].x >> 17;                     // unit 2^-14
+      norm += (unsigned)(l14 * l14);
+    }
+    return ok && (r < c + 8 || norm <= 265751040u);
+  };
   for (int c0 = 0; c0 < NB; c0 += 8) {
+    int2 (*l8)[10] = M.l8[(c0 >> 3) & 1];
+    // what the last eight columns left is looked over by two idle warps
+    if (c0 > 0 && t >= 2 * NB && t < 3 * NB && t - 2 * NB >= c0 - 8)
+      bad |= !fits(t - 2 * NB, c0 - 8, t - 2 * NB >= c0 + 8);
     // thread (row r, half hc): columns c0 + hc, + 2, + 4, + 6; a warp whose rows are
     // all done stays away
     if (t < 2 * NB && (t & (NB - 1)) >= (c0 & 32)) {
@@ -329,7 +356,7 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
           const double l = r == c0 + j ? M.diag[r] : a[i] * M.rinv[c0 + j];
           const long long v = c0 + j <= r ? to_fix(l, 63) : 0;
           if (c0 + j <= r) M.a[r][c0 + j] = v;
-          M.l8[r][j] = split56(v);
+          l8[r][j] = split56(v);
           M.inv[r][c0 + j] = l;            // the factor in fp64, for the halving
         }
       }
@@ -340,8 +367,8 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
     for (int i = 0; i < TRI; ++i) {
       if (t + WT * i >= rem * (rem + 1) / 2) continue;
       const int r = b0 + tr[i], c = b0 + tc[i];
-      const int4* lr = reinterpret_cast<const int4*>(M.l8[r]);
-      const int4* lc = reinterpret_cast<const int4*>(M.l8[c]);
+      const int4* lr = reinterpret_cast<const int4*>(l8[r]);
+      const int4* lc = reinterpret_cast<const int4*>(l8[c]);
       long long s1 = 0, s2 = 0;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -349,12 +376,16 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
         mac56(s1, s2, make_int2(x.x, x.y), make_int2(y.x, y.y));
         mac56(s1, s2, make_int2(x.z, x.w), make_int2(y.z, y.w));
       }
-      const long long v = M.a[r][c] - sum56(s1, s2);
+      const long long old = M.a[r][c], sum = sum56(s1, s2);
+      const long long v = (long long)((unsigned long long)old - (unsigned long long)sum);
+      bad |= ((old ^ sum) & (old ^ v)) < 0;
       M.a[r][c] = v;
       if (tc[i] < 8) M.cur[r][tc[i]] = from_fix(v, -63);
     }
+    if (rem == 0 && t >= 3 * NB - 8 && t < 3 * NB) bad |= !fits(t - 2 * NB, c0, false);
     workers_sync();
   }
+  if (bad) raise_status(status, BAKRON_ERR_NOT_SPD);
   // M.inv holds the factor (fp64).  The inverse: 8 x 8 diagonal blocks, a thread
   // per column ...
   double x8[8];
@@ -535,6 +566,14 @@ __device__ __forceinline__ uint32_t wide_int(uint32_t f) {
   const float x = __uint_as_float(f), h = fmaf(x, 0.5f, 12582912.f);
   const float rest = fmaf(h - 12582912.f, -2.f, x);
   return 2 * (__float_as_uint(h) - OZ_BIAS) + (__float_as_uint(rest + 12582912.f) - OZ_BIAS);
+}
+
+// The sum of a panel's products over 64 terms, 2^-14 as the unit, from its two leading
+// sums of digit products (the others add less than 49): up to this it is below 0.992
+// and fits; a positive definite matrix has at most 0.953 (15 650).
+constexpr float OZ_FIT = 16200.f;
+__device__ __forceinline__ float leading(uint32_t f0, uint32_t f1) {
+  return fabsf(fmaf(__uint_as_float(f1), 1.f / 256.f, __uint_as_float(f0)));
 }
 
 // Four 8-byte words, 32-byte aligned: whole sectors per lane.
@@ -739,6 +778,10 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
   long long acc[32];
   bool dead = false;
   constexpr bool one_chunk = MODE == OZ_TRSM || MODE == OZ_SYRK;
+  // the largest leading part of a sum, where sums are looked at: all of a TRSM's, and of a
+  // SYRK's the rows' norms, which bound the others
+  float most = 0.f;
+  const bool fit = MODE == OZ_TRSM || (MODE == OZ_SYRK && T.ra == T.rb && q == cg);
   static_assert(OT * 8 == 2 * WT, "two units of a per thread, two (or one) of b");
   for (int ch = 0; ch < (one_chunk ? 1 : T.kn); ++ch) {
     const int kk = NB * (T.k0 + ch);
@@ -793,6 +836,9 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
             tmem_ld8(ta + OT + c, r1);
             tmem_ld8(ta + 2 * OT + c, r2);
             tmem_wait_ld();
+            if (fit)
+#pragma unroll
+              for (int u = 0; u < 8; ++u) most = fmaxf(most, leading(r0[u], r1[u]));
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
               const uint32_t v = (((biased_int(r0[u]) << 8) + biased_int(r1[u])) << 8) + biased_int(r2[u]);
@@ -853,6 +899,7 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
   }
   __syncthreads();
   if (!*abort_flag) {
+    bool bad = most > OZ_FIT;
     // a warp's eight rows, four at a time (old values in flight together)
 #pragma unroll
     for (int rr = 0; rr < OT / WORKERS; rr += 4) {
@@ -876,12 +923,21 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
           const longlong2 v = *reinterpret_cast<const longlong2*>(st + r * OUT_LD + c);
           if constexpr (MODE == OZ_TRSM) {
             const int f0 = min(max(S.f[i0 + c] + 1, 0), 63), f1 = min(max(S.f[i0 + c + 1] + 1, 0), 63);
-            *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + i0 + c) =
-                make_longlong2((long long)((unsigned long long)v.x << f0),
-                               (long long)((unsigned long long)v.y << f1));
+            const longlong2 l = make_longlong2((long long)((unsigned long long)v.x << f0),
+                                               (long long)((unsigned long long)v.y << f1));
+            bad |= l.x >> f0 != v.x || l.y >> f1 != v.y;   // an entry of 1 or more
+            *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + i0 + c) = l;
           } else if constexpr (MODE == OZ_SYRK) {
+            // `left`: columns to the diagonal; above it C holds nothing yet
+            auto less = [&](long long o, long long x, int left) -> long long {
+              const long long y = (long long)(2 * (unsigned long long)x),
+                              w = (long long)((unsigned long long)o - (unsigned long long)y);
+              bad |= (left >= 0 && ((o ^ y) & (o ^ w)) < 0) || (left == 0 && w <= 0);
+              return w;
+            };
+            const int left = T.ra + r - T.rb - c;
             *reinterpret_cast<longlong2*>(S.C + (int64_t)(T.ra + r) * ld + T.rb + c) =
-                make_longlong2(old[j][cb].x - 2 * v.x, old[j][cb].y - 2 * v.y);
+                make_longlong2(less(old[j][cb].x, v.x, left), less(old[j][cb].y, v.y, left - 1));
           } else if constexpr (MODE == OZ_INV1) {
             const int er = S.xc[i0 + T.ra + r] - 62;
             *reinterpret_cast<double2*>((double*)S.C + (int64_t)(i0 + T.ra + r) * ld + i0 + arg + T.rb + c) =
@@ -894,6 +950,7 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
           }
         }
     }
+    if (bad) raise_status(P.status, BAKRON_ERR_NOT_SPD);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
