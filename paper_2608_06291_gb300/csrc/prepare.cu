@@ -14,7 +14,7 @@
 // Precision and units.  An fp32 factorisation has relative error ~kappa * 2^-24
 // (1e-5 at the condition numbers of the power-law Grams); error feedback
 // multiplies that into the pre-rounding values, too close to the 1e-4 tie band
-// on 4096-wide problems.  So the arithmetic is that of fp64 or better, but the
+// on 4096-wide problems.  So the factors have to be as good as fp64's, but the
 // GPU's fp64 units do 2 multiply-adds a cycle and SM (1.2 TFLOP/s in all), so
 // all products of matrices run on the tensor cores, on exact slices (Ozaki et
 // al. 2012, error-free transformations of matrix multiplication):
@@ -24,12 +24,15 @@
 //     ("Q63"), which loses less than an fp64 of the same matrix would.
 //   * An operand is cut into seven balanced base-256 digits, its upper 56 bits (Q63
 //     as it is; fp64 matrices relative to a power of two above each row's norm),
-//     each an fp16 integer of [-128, 127].  The 28 products of digit planes (i, j) with
-//     i + j <= 6 are exact in the tensor cores' fp32 accumulators over 64 terms
+//     each an fp16 integer of [-128, 127].  The 34 products of digit planes (i, j) with
+//     i + j <= 7 are exact in the tensor cores' fp32 accumulators over 64 terms
 //     (7 * 64 * 2^14 < 2^23); planes of equal i + j share one.  Their sum, shifted
-//     8 bits apart, is formed in 64-bit integers modulo 2^64, which is right where
-//     the result itself fits.  Dropped digit products are below 2^-53 of the product
-//     of the norms.
+//     8 bits apart (the last one rounded to the unit), is formed in 64-bit integers
+//     modulo 2^64, which is right where the result itself fits.  The digit products
+//     that are dropped are at most 2^-55 of the product of the norms per 64 terms and
+//     some 2^-61 typically, the operands' rounding to 56 bits 2^-52 and 2^-56.  (With
+//     the 28 products of i + j <= 6 the dropped ones were 2^-53 typically, and the
+//     factors five to fifteen times further off than an fp64 factorisation's.)
 //   * Of a positive definite matrix every result fits: entries of the factor and of
 //     the Schur complements, and sums over a factor's rows, are below 0.976
 //     (Cauchy-Schwarz).  Of another it need not, and a wrapped pivot could look
@@ -498,7 +501,7 @@ __global__ void __launch_bounds__(WT) k_prep_first(const PrepArgs P) {
 //   OZ_INV2  X21 = -X22 R^T
 // 128 x 128 tiles and 64-deep chunks, because the fourteen digit planes of one chunk
 // just fit shared memory.  What bounds a chunk: cutting the operands (6 to 9 thousand
-// cycles, integer work and the loads' latency), then 112 MMAs of 62 cycles and the
+// cycles, integer work and the loads' latency), then 136 MMAs of 62 cycles and the
 // sums, which partly run beside them (12 thousand); nothing of the next chunk can
 // start meanwhile.  9 to 10 us, against 20 to 28 with shifts by run-time counts and
 // a warp of its own for the MMAs.
@@ -654,10 +657,11 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
   constexpr int BN = MODE == OZ_TRSM ? NB : OT;        // columns of the MMAs
   constexpr uint32_t b_plane = BN * 128;
   unsigned char* pb = smem + SLICES * OPLANE;
-  // per chunk, the sums of digit products of equal weight s = 0 .. 6 are handed
-  // over as {0, 1, 2}, {3, 4}, {5, 6}; sum s sits in accumulator s & 3
-  uint64_t* accF = (uint64_t*)(smem + 2 * SLICES * OPLANE);   // [3] a group is complete
-  uint64_t* accE = accF + 3;                                   // group 0 has been read out
+  // per chunk, the sums of digit products of equal weight s = 0 .. 7 are handed
+  // over as {0, 1, 2}, {3, 4}, {5, 6}, {7}; sum s sits in accumulator s & 3
+  constexpr int GROUPS = 4;
+  uint64_t* accF = (uint64_t*)(smem + 2 * SLICES * OPLANE);   // [GROUPS] a group is complete
+  uint64_t* accE = accF + GROUPS;                              // group 0, then 1, has been read out
   uint64_t* done = accE + 1;
   uint32_t* tmem_slot = (uint32_t*)(done + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
@@ -672,7 +676,7 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
     return;
   }
   if (t == 0) {
-    for (int a = 0; a < 3; ++a) mbar_init(&accF[a], 1);
+    for (int a = 0; a < GROUPS; ++a) mbar_init(&accF[a], 1);
     mbar_init(accE, drains);
     mbar_init(done, 1);
     *abort_flag = 0;
@@ -765,13 +769,14 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
   auto issue = [&](auto s0, auto s1) {
 #pragma unroll
     for (int s = decltype(s0)::value; s <= decltype(s1)::value; ++s) {
+      const int first = max(0, s - SLICES + 1);
 #pragma unroll
-      for (int i = 0; i <= s; ++i) {
+      for (int i = first; i <= min(s, SLICES - 1); ++i) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           mma_bf16(tmem + (uint32_t)((s & 3) * OT), da + (uint64_t)(i * (OPLANE >> 4) + 2 * k),
                    db + (uint64_t)((s - i) * (b_plane >> 4) + 2 * k), idesc_f16(OT, BN),
-                   (i > 0 || k > 0) ? 1u : 0u);
+                   (i > first || k > 0) ? 1u : 0u);
       }
     }
   };
@@ -814,9 +819,9 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
     __syncwarp();
     if (warp < drains) {
       // sum s counts 2^(8 (6 - s)); modulo 2^64, so the first three only reach
-      // the upper word, and pairs of the others fit 32 bits
+      // the upper word, pairs of the others fit 32 bits, and the last is rounded
 #pragma unroll
-      for (int g = 0; g < 3; ++g) {
+      for (int g = 0; g < GROUPS; ++g) {
         int ok = dead ? 0 : 1;
         if (lane == 0 && !dead) {
           ok = oz_wait(&accF[g], (uint32_t)ch & 1u, P.spin_cycles, abort_flag) ? 1 : 0;
@@ -846,6 +851,16 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
                                 v - ((OZ_BIAS << 16) + (OZ_BIAS << 8) + OZ_BIAS)) << 32);
             }
           }
+        } else if (g == 3) {
+#pragma unroll
+          for (int c = 0; c < 32; c += 16) {
+            uint32_t r[16];
+            tmem_ld16(ta + 3 * OT + c, r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+              acc[c + u] += (int)(__float_as_uint(fmaf(__uint_as_float(r[u]), 1.f / 256.f, 12582912.f)) - OZ_BIAS);
+          }
         } else {
 #pragma unroll
           for (int c = 0; c < 32; c += 16) {
@@ -864,16 +879,21 @@ __global__ void __launch_bounds__(WT, 1) k_oz(const PrepArgs P, int arg) {
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        if (g == 0) {
+        if (g < 2) {
           __syncwarp();
           if (lane == 0) mbar_arrive(accE);
-          if (t == 0) {   // accumulators 0 .. 2 again
-            if (oz_wait(accE, (uint32_t)ch & 1u, P.spin_cycles, abort_flag)) {
+          if (t == 0) {   // accumulators 0 .. 2 again, then 3
+            if (oz_wait(accE, (uint32_t)g, P.spin_cycles, abort_flag)) {   // two phases a chunk
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              issue(Int<4>{}, Int<4>{});
-              mma_commit(&accF[1]);
-              issue(Int<5>{}, Int<6>{});
-              mma_commit(&accF[2]);
+              if (g == 0) {
+                issue(Int<4>{}, Int<4>{});
+                mma_commit(&accF[1]);
+                issue(Int<5>{}, Int<6>{});
+                mma_commit(&accF[2]);
+              } else {
+                issue(Int<7>{}, Int<7>{});
+                mma_commit(&accF[3]);
+              }
             } else if (!*abort_flag) {
               timed_out();
             }
