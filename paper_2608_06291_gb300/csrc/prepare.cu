@@ -241,22 +241,6 @@ __device__ __forceinline__ void workers_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(WT) : "memory");
 }
 
-// 1 / sqrt(p) for a normal p: the hardware's approximation and one cubic step.
-__device__ __forceinline__ double rsqrt64(double p) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
-  const double e = fma(-p * r, r, 1.0);
-  return fma(r * e, fma(0.375, e, 0.5), r);
-}
-
-// 1 / p the same way.
-__device__ __forceinline__ double rcp64(double p) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
-  const double e = fma(-p, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // An exponent above three times the largest magnitude of a warp's values (32
 // values of that exponent have a norm below one: sqrt(32) < 2^3 / 1.05).
 __device__ __forceinline__ int warp_exp8(double x) {
@@ -274,8 +258,8 @@ __device__ __forceinline__ int warp_exp8(double x) {
 // columns at a time in fp64: four warps, two threads a row with every other column
 // in registers; per column the entries are published, and a row's entry over the
 // pivot (a reciprocal) times the eight rows' entries updates what it holds, so that
-// the square roots wait for the end, a lane each (6 fp64 instructions a column; a
-// thread per row with 1 / sqrt inside each column took 10).  Then one update of the
+// the square roots wait for the end, a lane each (with the quotient itself in place
+// of the reciprocal both sides 4096 took 12.23 ms, not 10.47).  Then one update of the
 // rest by all warps on split 56-bit values (three 32 x 32 + 64 multiply-adds each).
 // The inverse by halving: 8 x 8 blocks and the first two levels in fp64, the last
 // in integers.
@@ -335,7 +319,7 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
         if (j == 7) break;
         double p = M.col[j][c0 + j];
         if (!(p > 0.0)) p = 1.0;
-        const double lr = M.col[j][r] * rcp64(p);
+        const double lr = M.col[j][r] * (1.0 / p);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           if (2 * i + hc > j) a[i] = fma(-lr, M.col[j][c0 + 2 * i + hc], a[i]);
@@ -346,7 +330,7 @@ __device__ void potrf_block(const PrepSide& S, int k0, PotrfSmem& M, int* status
           raise_status(status, BAKRON_ERR_NOT_SPD);
           p = 1.0;
         }
-        const double ri = rsqrt64(p);
+        const double ri = rsqrt(p);
         M.rinv[r] = ri;
         M.diag[r] = p * ri;
         S.ldiag[k0 + r] = p * ri;
