@@ -215,7 +215,10 @@ int bakron_solve_with_grid(const void* W, int wdtype, int m, int n, int64_t ldw,
  *   workspace device scratch of at least bakron_gram_workspace_bytes(d, 1,
  *            w != NULL) bytes; the samples are processed in chunks of as many
  *            as fit (bakron_gram_workspace_bytes(d, c, weighted) holds c), so
- *            a larger workspace means fewer, larger launches
+ *            a larger workspace means fewer, larger launches.  bf16 samples
+ *            without weights whose rows can be read in place (d a multiple of
+ *            64, rows 16-byte aligned) need none of it for themselves; their
+ *            chunks are as long, or 5 k^(2/3) samples if that is more
  *   sync     nonzero: synchronise `stream` and return the device status
  * On the tensor cores (tcgen05), FP32-accurate.  bf16 samples without
  * weights: kind::f16 MMAs on the bf16 values (products exact in fp32), each
