@@ -411,10 +411,12 @@ __global__ void __launch_bounds__(GR_THREADS, 1)
 }
 
 // G's lower triangle and its mirror from the parts of k_gram (splits > 1),
-// added in the order of the splits: 32 x 32 entries per block.
+// added in the order of the splits: 32 x 32 entries per block.  After a time-out
+// parts are missing, and G is left as it is.
 template <int BN>
 __global__ void __launch_bounds__(256) k_gram_reduce(const GramParams P) {
   __shared__ float t[32][33];
+  if (*P.status != BAKRON_OK) return;         // uniform: k_gram is done
   int rb, cb;
   gram_block<BN>(blockIdx.x, rb, cb);
   const int r0 = 32 * (blockIdx.y / (BN / 32)), c0 = 32 * (blockIdx.y % (BN / 32));
