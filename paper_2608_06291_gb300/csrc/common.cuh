@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <mutex>
+
 #include "../../include/bakron.h"
 
 namespace bakron {
@@ -208,6 +210,32 @@ __device__ __forceinline__ void mma_tf32_16x8x8(float (&d)[4], const uint32_t (&
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+
+// Runs `set` once per device, for what belongs to the current device (kernel
+// attributes); again where it failed.  Safe from several threads.
+class OncePerDevice {
+ public:
+  template <typename F>
+  cudaError_t on(int dev, const F& set) {
+    if (dev < 0 || dev >= MAX_DEVICES) return set();
+    std::lock_guard<std::mutex> lk(mu_);
+    if (done_[dev]) return cudaSuccess;
+    const cudaError_t e = set();
+    done_[dev] = e == cudaSuccess;
+    return e;
+  }
+  template <typename F>
+  cudaError_t operator()(const F& set) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? on(dev, set) : e;
+  }
+
+ private:
+  static constexpr int MAX_DEVICES = 64;
+  std::mutex mu_;
+  bool done_[MAX_DEVICES] = {};
+};
 
 // Device status word (first int of every workspace).  Kernels only ever raise
 // it with atomicMax-free writes of a nonzero code; the host reads and clears.

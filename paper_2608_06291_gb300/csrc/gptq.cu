@@ -21,7 +21,6 @@
 
 #include <algorithm>
 #include <cstdlib>
-#include <mutex>
 
 #include "common.cuh"
 #include "profile.cuh"
@@ -307,13 +306,11 @@ int gptq_impl(const void* W, int wdt, int m, int n, int64_t ldw, const void* fac
   SolveLayout sl(m, n);
   char* ws = (char*)workspace;
   const char* f = (const char*)factors;
-  static std::once_flag attr_once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(k_gptq_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(GptqSmem));
-  });
-  if (attr_err != cudaSuccess) return BAKRON_ERR_CUDA;
+  static OncePerDevice attrs;
+  BK_CUDA_OK(attrs([] {
+    return cudaFuncSetAttribute(k_gptq_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(GptqSmem));
+  }));
   GqRun r;
   r.s = s;
   r.rc = BAKRON_OK;

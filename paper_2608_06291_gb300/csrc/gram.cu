@@ -38,7 +38,6 @@
 #include <stdlib.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "tc_gemm.cuh"
@@ -564,21 +563,19 @@ constexpr int GRAM_MAX_D = 1 << 16;
 constexpr int SM_COUNT = 152;
 
 cudaError_t gram_attrs() {
-  static std::mutex mu;
-  static bool done = false;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done) return cudaSuccess;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_gram<OP_BF16_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           GramShape<OP_BF16_MN>::smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gram<OP_BF16_K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             GramShape<OP_BF16_K>::smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gram<OP_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             GramShape<OP_TF32>::smem);
-  if (e == cudaSuccess) done = true;
-  return e;
+  static OncePerDevice once;
+  return once([] {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_gram<OP_BF16_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             GramShape<OP_BF16_MN>::smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_gram<OP_BF16_K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               GramShape<OP_BF16_K>::smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_gram<OP_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               GramShape<OP_TF32>::smem);
+    return e;
+  });
 }
 
 // A tiled tensor map with the 128-byte swizzle and boxes inside 128-byte rows.

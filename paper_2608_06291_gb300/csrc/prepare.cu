@@ -51,8 +51,6 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <mutex>
-
 #include "common.cuh"
 #include "tc_gemm.cuh"
 #include "tcgen05.cuh"
@@ -1067,22 +1065,20 @@ __global__ void __launch_bounds__(256) k_assemble(const PrepSide S, float* L, fl
 }
 
 cudaError_t prep_attrs() {
-  static std::mutex mu;
-  static bool done = false;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_prep_first, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(PotrfSmem));
-  auto set = [&](const void* f) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
-  };
-  set((const void*)k_oz<OZ_TRSM>);
-  set((const void*)k_oz<OZ_SYRK>);
-  set((const void*)k_oz<OZ_INV1>);
-  set((const void*)k_oz<OZ_INV2>);
-  if (e == cudaSuccess) done = true;
-  return e;
+  static OncePerDevice once;
+  return once([] {
+    cudaError_t e = cudaFuncSetAttribute(k_prep_first, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(PotrfSmem));
+    auto set = [&](const void* f) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
+    };
+    set((const void*)k_oz<OZ_TRSM>);
+    set((const void*)k_oz<OZ_SYRK>);
+    set((const void*)k_oz<OZ_INV1>);
+    set((const void*)k_oz<OZ_INV2>);
+    return e;
+  });
 }
 
 // One side from where its matrices are (PrepareScratch).

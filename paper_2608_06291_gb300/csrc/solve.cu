@@ -2067,26 +2067,24 @@ static void leaf_block(SolveArgs& a, int k, int l) {
 }
 
 // Dynamic shared memory of the leaf and subtree kernels above the 48 KB
-// default, set once per process.
+// default, set once per device.
 static cudaError_t ensure_leaf_attrs() {
-  static std::mutex mu;
-  static bool done = false;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done) return cudaSuccess;
-  const int sm = (int)sizeof(LeafSmem), ss = (int)sizeof(SubtreeSmem);
-  cudaError_t e = set_leaf_smem<0>(sm);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(StripSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_strips_heads, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(StripSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_subtree, cudaFuncAttributeMaxDynamicSharedMemorySize, ss);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_leaf_flow, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) done = true;
-  return e;
+  static OncePerDevice once;
+  return once([] {
+    const int sm = (int)sizeof(LeafSmem), ss = (int)sizeof(SubtreeSmem);
+    cudaError_t e = set_leaf_smem<0>(sm);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_strips, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(StripSmem));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_strips_heads, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(StripSmem));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_subtree, cudaFuncAttributeMaxDynamicSharedMemorySize, ss);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_leaf_flow, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    return e;
+  });
 }
 
 static void band(SolveArgs& a, int k, int h, int l) {

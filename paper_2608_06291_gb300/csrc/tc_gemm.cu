@@ -901,22 +901,19 @@ bool make_map_pair(CUtensorMap* map, const float* hi, const float* lo, int64_t r
   return r == CUDA_SUCCESS;
 }
 
-bool g_attr_done = false;
-std::mutex g_attr_mu;
-
 cudaError_t ensure_attr() {
-  std::lock_guard<std::mutex> lk(g_attr_mu);
-  if (g_attr_done) return cudaSuccess;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_tc_band<V_BAND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           SMEM_BYTES);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_band<V_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             PAIR_SMEM_BYTES);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_heads, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  if (e == cudaSuccess) g_attr_done = true;
-  return e;
+  static OncePerDevice once;
+  return once([] {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_tc_band<V_BAND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_tc_band<V_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               PAIR_SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_tc_heads, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    return e;
+  });
 }
 
 // The paired kernel: clusters of two CTAs along x, with programmatic
