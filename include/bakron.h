@@ -75,8 +75,10 @@ size_t bakron_workspace_bytes(int m, int n);
  *   damp     >= 0, relative diagonal damping
  *   factors  device, bakron_factors_bytes(m, n) bytes, written
  *   workspace device, >= bakron_workspace_bytes(m, n) bytes, scratch
- * Synchronises `stream` at the end and returns BAKRON_ERR_NOT_SPD if a pivot
- * of the damped A or B was not positive (factors are then undefined).
+ * Synchronises `stream` at the end and returns BAKRON_ERR_NOT_SPD if the damped
+ * A or B is not positive definite or not finite (factors are then undefined), or
+ * BAKRON_ERR_TIMEOUT if a bounded device wait ran out.  The factors are no
+ * further off than an fp64 factorisation's rounded to fp32 (by norm).
  */
 int bakron_prepare(const float* A, const float* B, int m, int n, float damp,
                    void* factors, void* workspace, size_t workspace_bytes,

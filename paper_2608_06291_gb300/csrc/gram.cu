@@ -28,7 +28,8 @@
 // samples of 4096 features 0.54 -> 0.24 ms (1.13 PFLOP/s), of which 0.07 was the
 // transposed copy that MN-major operands need no more.  Blocks too few for the SMs
 // are split along the samples (gram_splits), the parts summed in order by
-// k_gram_reduce (5000 weighted fp32 samples of 1531 features: 120 -> 75 us).
+// k_gram_reduce (5000 weighted fp32 samples of 1531 features: 120 -> 75 us).  The bf16
+// forms' epilogue threads hold 128 sums each and spill 58 bytes.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -44,7 +44,8 @@
 // integers.
 //
 // Measured on GB300, both sides 4096: 160.2 ms with the products on the fp64 units,
-// 9.3 so; 1531 + 1000: 26.7 -> 2.7.
+// 10.5 so; 1531 + 1000: 26.7 -> 3.1.  (Of the 10.5, 0.65 are the last six digit
+// products, 0.25 the looks at what fits, 0.27 CUDA's reciprocal and root.)
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -484,9 +485,10 @@ __global__ void __launch_bounds__(WT) k_prep_first(const PrepArgs P) {
 // 128 x 128 tiles and 64-deep chunks, because the fourteen digit planes of one chunk
 // just fit shared memory.  What bounds a chunk: cutting the operands (6 to 9 thousand
 // cycles, integer work and the loads' latency), then 136 MMAs of 62 cycles and the
-// sums, which partly run beside them (12 thousand); nothing of the next chunk can
-// start meanwhile.  9 to 10 us, against 20 to 28 with shifts by run-time counts and
-// a warp of its own for the MMAs.
+// sums, which partly run beside them (some 14 thousand); nothing of the next chunk can
+// start meanwhile.  10 to 11.5 us, against 20 to 28 with shifts by run-time counts and
+// a warp of its own for the MMAs.  Sixteen warps leave 128 registers a thread, over
+// which OZ_INV1, with its strided loads, spills 160 bytes.
 enum OzMode { OZ_TRSM, OZ_SYRK, OZ_INV1, OZ_INV2 };
 
 // Seven digits of eight values (Q63) to the planes: 16 bytes of a row each, in

@@ -558,9 +558,9 @@ __device__ __forceinline__ void wave_chain(SM& S, const float (*LA0)[KM], int64_
     S.Ebr[d & 3][p & (TILE - 1)] = e;    // rows off the tile get a zero
   };
   // the grid and the sub-diagonal L^B of the next interval's entries are
-  // loaded one interval ahead; two intervals per loop iteration (in k_strips
-  // 173 cycles a step, against 188 with one and 194 with three or six: the three
-  // teams' loops share the instruction caches)
+  // loaded one interval ahead; two intervals per loop iteration (cycles a step,
+  // warm: 167 to 181 in k_strips, where one took 188 and three or six 194 beside the
+  // other teams, whose loops share the instruction caches; 176 in k_leaf, three 181)
   float4 g0 = S.Srzl[(0 - q) & (TILE - 1)][q], g1 = S.Srzl[(1 - q) & (TILE - 1)][q];
   float4 lb0 = S.Lsub[(0 - q) & (TILE - 1)], lb1 = S.Lsub[(1 - q) & (TILE - 1)];
   leaf_sync();   // the helpers' pre of steps 0 and 1
